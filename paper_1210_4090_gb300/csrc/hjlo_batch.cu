@@ -561,7 +561,7 @@ hjlo_status hjlo_batch_run(hjlo_batch *b, void *const *u, const double *const *V
                 it.hoff = ax.hoff;
                 it.dhi = (int)ax.dhi;
                 if (ax.layout == LAYOUT_CONTIG)
-                    it.use_tma = (((uintptr_t)u[i] & 15) == 0) && (((ax.N * b->esize) & 15) == 0);
+                    it.use_tma = contig_tma(ax, b->esize, u[i]) ? 1 : 0;
                 else
                     it.use_tma = encode_strided(ax, b->esize, u[i], &it.tmap) ? 1 : 0;
             }

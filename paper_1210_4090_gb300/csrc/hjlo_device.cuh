@@ -75,6 +75,8 @@ struct PassParams {
     double kmax;              // max |k| over the window
     double curv;              // lower bound of the min second difference of k (inf if weff < 3)
     int off_u, off_fx, off_kfx, off_t, off_k64, off_misc;  // shared memory offsets (bytes)
+    int off_kp, off_q, qcap;  // banded search: pivot table, queues of flagged rows and their length
+    int dense;                // MONGE: 0, or the banded search's rows per segment (hjlo_dense.cuh)
     long long wait_ns;        // bound on the first mbarrier wait of a tile
     int test_extra_tx;        // test knob: bytes the barrier expects beyond the copy (0 in use)
     double hscale;            // hv_scaled: potential term fl(m - fl(hscale * hv[x]))
@@ -336,8 +338,9 @@ __device__ __forceinline__ Tile<LAYOUT> tile_of(const PassParams &p, long long t
         long long rem = p.outer - l0;
         t.valid = (int)(rem < p.C ? rem : p.C);
     } else {
-        long long o = tile / p.tiles_per_outer;
-        long long in0 = (tile - o * p.tiles_per_outer) << p.log2C;
+        // 32-bit division: a launch has fewer than 2^31 tiles
+        const unsigned o = (unsigned)tile / (unsigned)p.tiles_per_outer;
+        const long long in0 = (long long)((unsigned)tile - o * (unsigned)p.tiles_per_outer) << p.log2C;
         t.base = o * p.N * p.inner + in0;
         t.lstride = 1;
         t.pstride = p.inner;
@@ -527,48 +530,209 @@ __device__ __forceinline__ void count_edges(const PassParams &p, int edges)
     if ((threadIdx.x & 31) == 0 && we) atomicAdd(&p.counters[CNT_EDGE], (unsigned long long)we);
 }
 
-// Write-back of rows i = i0, i0 + step, ... < i1 of one contiguous line: the
-// exact value fl(u[src] + k[d]) at the recorded argmin, minus fl(h V) when
-// the pass carries the potential term, stored (binary32: rounded), with the
-// optional argmin.  Four rows per thread at a time, their potential-term
-// loads issued together.  Returns how many of the rows' argmins sit on the
-// window's edge.
-template <typename T, typename OFF>
-__device__ __forceinline__ int write_rows_contig(const PassParams &p, const T *lu, const OFF *lt,
-                                                  const double *kr64, T *dst, long long xb, int i0, int i1, int step)
+// Write-back of rows i = i0, i0 + step, ... < i1 of one line of the staged
+// tile (lu: the line's first value, positions 2^sh values apart; element x0 of
+// the grid is row i0's, xs elements on to the next): the exact value
+// fl(u[src] + k[d]) at the recorded argmin, minus fl(h V) when the pass
+// carries the potential term (HV), stored (binary32: rounded), with the
+// optional argmin (AM).  Four rows per thread at a time, their loads issued
+// together; the source's position wraps by an unsigned minimum.  Returns how
+// many of the rows' argmins sit on a partial window's edge.
+template <typename T, typename OFF, bool HV, bool AM>
+__device__ __forceinline__ int write_rows(const PassParams &p, const T *lu, int sh, const OFF *lt, const double *kr64,
+                                          int i0, int i1, int step, long long x0, long long xs)
 {
-    const int N = (int)p.N;
-    T *gd = dst + xb;
-    const double *gh = p.hv ? p.hv + xb : nullptr;
-    int32_t *ga = p.amin ? p.amin + xb : nullptr;
+    const int N = (int)p.N, weff = p.weff;
+    const int hs = step < N ? step : step % N;
+    int h = i0 % N + p.hoff;                                   // (i + hoff) mod N
+    h = (int)min((unsigned)h, (unsigned)(h - N));
+    T *gd = reinterpret_cast<T *>(p.dst) + x0;
+    const double *gh = HV ? p.hv + x0 : nullptr;
+    int32_t *ga = AM ? p.amin + x0 : nullptr;
     int edges = 0;
+    auto one = [&](int t, int hh) -> double {
+        const int pw = hh + t;                                 // < 2 N
+        const int pos = (int)min((unsigned)pw, (unsigned)(pw - N));
+        return __dadd_rn(widen(lu[pos << sh]), kr64[t]);
+    };
+    auto next = [&](int hh) -> int {
+        hh += hs;
+        return (int)min((unsigned)hh, (unsigned)(hh - N));
+    };
     int i = i0;
     for (; i + 3 * step < i1; i += 4 * step) {
-        double hvb[4];
-#pragma unroll
-        for (int b = 0; b < 4; ++b) hvb[b] = gh ? __ldg(gh + i + b * step) : 0.0;
+        double hvb[4], m[4];
+        int t[4];
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
-            const int ii = i + b * step;
-            const int t = lt[ii];
-            const int pos = wrapN(ii + t + p.hoff, N);
-            double m = __dadd_rn(widen(lu[pos]), kr64[t]);
-            if (gh) m = __dsub_rn(m, p.hv_scaled ? __dmul_rn(p.hscale, hvb[b]) : hvb[b]);
-            store_val(gd + ii, m);
-            if (ga) ga[ii] = p.dhi - t;
-            edges += on_edge(t, p.weff);
+            if (HV) hvb[b] = __ldg(gh + b * xs);
+            t[b] = lt[i + b * step];
         }
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            m[b] = one(t[b], h);
+            h = next(h);
+            edges += on_edge(t[b], weff);
+        }
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            if (HV) m[b] = __dsub_rn(m[b], p.hv_scaled ? __dmul_rn(p.hscale, hvb[b]) : hvb[b]);
+            store_val(gd + b * xs, m[b]);
+            if (AM) ga[b * xs] = p.dhi - t[b];
+        }
+        gd += 4 * xs;
+        if (HV) gh += 4 * xs;
+        if (AM) ga += 4 * xs;
     }
     for (; i < i1; i += step) {
         const int t = lt[i];
-        const int pos = wrapN(i + t + p.hoff, N);
-        double m = __dadd_rn(widen(lu[pos]), kr64[t]);
-        if (gh) m = __dsub_rn(m, p.hv_scaled ? __dmul_rn(p.hscale, gh[i]) : gh[i]);
-        store_val(gd + i, m);
-        if (ga) ga[i] = p.dhi - t;
-        edges += on_edge(t, p.weff);
+        double m = one(t, h);
+        h = next(h);
+        if (HV) m = __dsub_rn(m, p.hv_scaled ? __dmul_rn(p.hscale, *gh) : *gh);
+        store_val(gd, m);
+        if (AM) *ga = p.dhi - t;
+        edges += on_edge(t, weff);
+        gd += xs;
+        if (HV) gh += xs;
+        if (AM) ga += xs;
     }
-    return edges;
+    return p.edge ? edges : 0;
+}
+
+template <typename T, typename OFF>
+__device__ __forceinline__ int write_rows(const PassParams &p, const T *lu, int sh, const OFF *lt, const double *kr64,
+                                          int i0, int i1, int step, long long x0, long long xs)
+{
+    if (p.amin)
+        return p.hv ? write_rows<T, OFF, true, true>(p, lu, sh, lt, kr64, i0, i1, step, x0, xs)
+                    : write_rows<T, OFF, false, true>(p, lu, sh, lt, kr64, i0, i1, step, x0, xs);
+    return p.hv ? write_rows<T, OFF, true, false>(p, lu, sh, lt, kr64, i0, i1, step, x0, xs)
+                : write_rows<T, OFF, false, false>(p, lu, sh, lt, kr64, i0, i1, step, x0, xs);
+}
+
+// Rows i0, i0 + step, ... < i1 of a contiguous line whose row 0 is element xb.
+template <typename T, typename OFF>
+__device__ __forceinline__ int write_rows_contig(const PassParams &p, const T *lu, const OFF *lt, const double *kr64,
+                                                 long long xb, int i0, int i1, int step)
+{
+    return write_rows<T, OFF>(p, lu, 0, lt, kr64, i0, i1, step, xb + i0, step);
+}
+
+// A tile of strided lines (line index fastest).
+template <typename T, typename OFF>
+__device__ __forceinline__ int write_rows_strided(const PassParams &p, const Tile<LAYOUT_STRIDED> &tl, const T *su,
+                                                  const OFF *tt, const double *kr64)
+{
+    const int l = threadIdx.x & (p.C - 1), i0 = threadIdx.x >> p.log2C, step = blockDim.x >> p.log2C;
+    if (l >= tl.valid) return 0;
+    return write_rows<T, OFF>(p, su + l, p.log2C, tt + l * p.tp, kr64, i0, (int)p.N, step,
+                              tl.base + l + (long long)i0 * tl.pstride, (long long)step * tl.pstride);
+}
+
+// One element into shared memory without waiting (cp.async).
+template <typename T>
+__device__ __forceinline__ void copy_async(T *dst, const T *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_addr(dst)), "l"(src), "n"(sizeof(T)) : "memory");
+}
+
+// Starts staging a tile's lines in shared memory: TMA where the launch allows
+// it (the last bytes short of 16 of contiguous lines by plain stores), else
+// asynchronous copies of single elements, so that all of a thread's loads are
+// in flight at once.  `tmap`: the 3D TMA descriptor of the source for strided
+// lines (unused otherwise).  The barrier's phase ends with the TMA copies.
+template <typename T, int LAYOUT>
+__device__ __forceinline__ void stage_issue(const CUtensorMap *tmap, const PassParams &p, long long tile, T *su,
+                                            uint64_t *bar)
+{
+    const int tid = threadIdx.x, nthr = blockDim.x;
+    const int N = (int)p.N, C = p.C;
+    const T *src = reinterpret_cast<const T *>(p.src);
+    const Tile<LAYOUT> tl = tile_of<LAYOUT>(p, tile);
+    if (p.use_tma) {
+        if (LAYOUT == LAYOUT_CONTIG) {
+            const unsigned n = (unsigned)(tl.valid * N), bytes = n * (unsigned)sizeof(T), whole = bytes & ~15u;
+            if (tid == 0) {
+                mbar_arrive_expect_tx(bar, whole + (uint32_t)p.test_extra_tx);
+                if (whole) tma_bulk_load(su, src + tl.base, whole, bar);
+            }
+            const unsigned k = whole / (unsigned)sizeof(T) + (unsigned)tid;
+            if (k < n) su[k] = src[tl.base + k];
+        } else if (tid == 0) {
+            const uint32_t bytes = (uint32_t)(p.nbox * p.by * C * (int)sizeof(T));
+            mbar_arrive_expect_tx(bar, bytes + (uint32_t)p.test_extra_tx);
+            const unsigned o = (unsigned)tile / (unsigned)p.tiles_per_outer;
+            const int x0 = (int)(((unsigned)tile - o * (unsigned)p.tiles_per_outer) << p.log2C);
+            for (int b = 0; b < p.nbox; ++b)
+                tma_tensor_load_3d(su + (long long)b * p.by * C, tmap, x0, b * p.by, (int)o, bar);
+        }
+    } else if (LAYOUT == LAYOUT_CONTIG && p.vN) {
+        // row blocks: gather each block's window span from its real line
+        // (N <= vN, so one wrap at most)
+        for (int l = 0; l < tl.valid; ++l) {
+            const long long vl = (tile << p.log2C) + l;
+            const long long rl = ((vl | p.vblocks) >> 32) ? vl / p.vblocks
+                                                          : (long long)((unsigned)vl / (unsigned)p.vblocks);
+            const T *ls = src + rl * p.vN;
+            const unsigned vN = (unsigned)p.vN;                // a line has at most 2^24 points
+            unsigned s0 = (unsigned)(vl - rl * p.vblocks) * (unsigned)p.vR + (unsigned)p.vhoff;   // < 2 vN
+            s0 = min(s0, s0 - vN);
+            for (int i = tid; i < N; i += nthr) {
+                const unsigned q = s0 + (unsigned)i;
+                copy_async(su + l * N + i, ls + min(q, q - vN));
+            }
+        }
+    } else if (LAYOUT == LAYOUT_CONTIG) {
+        const int n = tl.valid * N;
+        for (int i = tid; i < n; i += nthr) copy_async(su + i, src + tl.base + i);
+    } else {
+        const int l = tid & (C - 1), step = nthr >> p.log2C;
+        int i = tid >> p.log2C;
+        const T *g = src + tl.base + l + (long long)i * tl.pstride;
+        if (l < tl.valid)
+            for (; i < N; i += step, g += (long long)step * tl.pstride) copy_async(su + (i << p.log2C) + l, g);
+    }
+    // the potential term of a contiguous tile is read at the very end: start
+    // moving it towards L2 now, behind the search
+    if (LAYOUT == LAYOUT_CONTIG && p.hv && !p.vN && tid == nthr - 1)
+        prefetch_l2(p.hv + tl.base, (unsigned long long)tl.valid * N * sizeof(double));
+}
+
+// Waits for what the thread and the block have started (a block barrier: what
+// the threads wrote to shared memory before it is visible after it).  False
+// when a TMA copy did not land in time (flagged).
+__device__ __forceinline__ bool stage_wait(const PassParams &p, uint64_t *bar, uint32_t parity)
+{
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    if (!p.use_tma) {
+        __syncthreads();
+        return true;
+    }
+    // one thread waits, the others at the barrier; then each looks once
+    const bool ok = (threadIdx.x != 0) || mbar_wait_bounded(bar, parity, p.wait_ns);
+    if (__syncthreads_or(!ok) || !mbar_wait_bounded(bar, parity, p.wait_ns)) {
+        // the copy did not land in time: flag it, give it one more bounded
+        // wait so nothing is still writing our shared memory, and leave
+        if (threadIdx.x == 0) atomicOr(p.flags, FLAG_TIMEOUT);
+        mbar_wait_bounded(bar, parity, 500000000LL);
+        return false;
+    }
+    return true;
+}
+
+// Stages one tile and the kernel table; false as stage_wait.
+template <typename T, int LAYOUT>
+__device__ __forceinline__ bool stage_tile(const CUtensorMap *tmap, const PassParams &p, long long tile, T *su,
+                                           double *kr64, uint64_t *bar)
+{
+    if (threadIdx.x == 0) {
+        mbar_init(bar, 1);
+        fence_mbar_init();
+    }
+    __syncthreads();
+    stage_issue<T, LAYOUT>(tmap, p, tile, su, bar);
+    for (int i = threadIdx.x; i < p.weff; i += blockDim.x) copy_async(kr64 + i, p.kr64 + i);
+    return stage_wait(p, bar, 0);
 }
 
 // Per-line facts of the fixed-point screen, in shared memory.
@@ -601,69 +765,13 @@ __device__ __forceinline__ void pass_tile(const CUtensorMap *tmap, const PassPar
     const int tid = threadIdx.x, nthr = blockDim.x;
     const int N = (int)p.N, C = p.C, weff = p.weff;
     const Tile<LAYOUT> tl = tile_of<LAYOUT>(p, tile);
-    const T *src = reinterpret_cast<const T *>(p.src);
 
     // ---- stage the tile
-    if (tid == 0) {
-        mbar_init(bar, 1);
-        fence_mbar_init();
-    }
     if (ALGO == KALGO_MONGE && tid < C) {
         li[tid].kmin = 0x7fffffff;
         li[tid].kmax = (int)0x80000000;
     }
-    __syncthreads();
-    if (p.use_tma) {
-        if (tid == 0) {
-            if (LAYOUT == LAYOUT_CONTIG) {
-                uint32_t bytes = (uint32_t)((long long)tl.valid * N * (long long)sizeof(T));
-                mbar_arrive_expect_tx(bar, bytes + (uint32_t)p.test_extra_tx);
-                tma_bulk_load(su, src + tl.base, bytes, bar);
-            } else {
-                uint32_t bytes = (uint32_t)(p.nbox * p.by * C * (int)sizeof(T));
-                mbar_arrive_expect_tx(bar, bytes + (uint32_t)p.test_extra_tx);
-                long long o = tile / p.tiles_per_outer;
-                int x0 = (int)((tile - o * p.tiles_per_outer) << p.log2C);
-                for (int b = 0; b < p.nbox; ++b)
-                    tma_tensor_load_3d(su + (long long)b * p.by * C, tmap, x0, b * p.by, (int)o, bar);
-            }
-        }
-    } else if (LAYOUT == LAYOUT_CONTIG && p.vN) {
-        // row blocks: gather each block's window span from its real line
-        // (N <= vN, so one wrap at most)
-        for (int l = 0; l < tl.valid; ++l) {
-            const long long vl = (tile << p.log2C) + l;
-            const long long rl = vl / p.vblocks;
-            const T *ls = src + rl * p.vN;
-            const long long s0 = ((vl - rl * p.vblocks) * p.vR + p.vhoff) % p.vN;
-            for (int i = tid; i < N; i += nthr) {
-                long long q = s0 + i;
-                q = (q >= p.vN) ? q - p.vN : q;
-                su[l * N + i] = ls[q];
-            }
-        }
-    } else {
-        for (int l = 0; l < tl.valid; ++l)
-            for (int i = tid; i < N; i += nthr)
-                su[uidx<LAYOUT>(p, l, i)] = src[tl.base + l * tl.lstride + (long long)i * tl.pstride];
-    }
-    // the potential term of a contiguous tile is read at the very end: start
-    // moving it towards L2 now, behind the search
-    if (LAYOUT == LAYOUT_CONTIG && p.hv && !p.vN && tid == nthr - 1)
-        prefetch_l2(p.hv + tl.base, (unsigned long long)tl.valid * N * sizeof(double));
-    for (int i = tid; i < weff; i += nthr) kr64[i] = p.kr64[i];
-    if (p.use_tma) {
-        bool ok = mbar_wait_bounded(bar, 0, p.wait_ns);
-        if (__syncthreads_or(!ok)) {
-            // the copy did not land in time: flag it, give it one more bounded
-            // wait so nothing is still writing our shared memory, and leave
-            if (tid == 0) atomicOr(p.flags, FLAG_TIMEOUT);
-            mbar_wait_bounded(bar, 0, 500000000LL);
-            return;
-        }
-    } else {
-        __syncthreads();
-    }
+    if (!stage_tile<T, LAYOUT>(tmap, p, tile, su, kr64, bar)) return;
 
     const int lane = tid & 31, warp = tid >> 5;
 
@@ -915,7 +1023,6 @@ __device__ __forceinline__ void pass_tile(const CUtensorMap *tmap, const PassPar
             // stay inside the warp after P2), so each warp writes its own rows
             // back as soon as it is done: no block barrier, coalesced stores.
             __syncwarp();
-            T *dst = reinterpret_cast<T *>(p.dst);
             const int nl = (lpl >= 32) ? 1 : (32 >> p.log2lpl);     // lines held by this warp
             int edges = 0;
             for (int k = 0; k < nl; ++k) {
@@ -934,7 +1041,7 @@ __device__ __forceinline__ void pass_tile(const CUtensorMap *tmap, const PassPar
                     xb = rb.base;
                     r1 = min(r1, rb.rows);
                 }
-                edges += write_rows_contig<T, OFF>(p, su + l * N, tt + l * p.tp, kr64, dst, xb, r0 + lane, r1, 32);
+                edges += write_rows_contig<T, OFF>(p, su + l * N, tt + l * p.tp, kr64, xb, r0 + lane, r1, 32);
             }
             count_edges(p, edges);
             return;
@@ -973,9 +1080,8 @@ __device__ __forceinline__ void pass_tile(const CUtensorMap *tmap, const PassPar
     __syncthreads();
 
     // ---- exact values, potential term, stores (coalesced order)
-    T *dst = reinterpret_cast<T *>(p.dst);
     int edges = 0;
-    if (LAYOUT == LAYOUT_CONTIG) {
+    if constexpr (LAYOUT == LAYOUT_CONTIG) {
         const int lanes = nthr >> p.log2C;              // threads per line
         const int l = tid / lanes, sub = tid - l * lanes;
         if (l < tl.valid) {
@@ -986,27 +1092,10 @@ __device__ __forceinline__ void pass_tile(const CUtensorMap *tmap, const PassPar
                 xb = rb.base;
                 rows = rb.rows;
             }
-            edges = write_rows_contig<T, OFF>(p, su + l * N, tt + l * p.tp, kr64, dst, xb, sub, rows, lanes);
+            edges = write_rows_contig<T, OFF>(p, su + l * N, tt + l * p.tp, kr64, xb, sub, rows, lanes);
         }
     } else {
-        const int l = tid & (C - 1);
-        if (l < tl.valid) {
-            const int step = nthr >> p.log2C;
-            const OFF *lt = tt + l * p.tp;
-            const long long xb = tl.base + l;
-            const long long xs = (long long)step * tl.pstride;
-            int i = tid >> p.log2C;
-            long long x = xb + (long long)i * tl.pstride;
-            for (; i < N; i += step, x += xs) {
-                const int t = lt[i];
-                const int pos = wrapN(i + t + p.hoff, N);
-                double m = __dadd_rn(widen(su[(pos << p.log2C) + l]), kr64[t]);
-                if (p.hv) m = __dsub_rn(m, p.hv_scaled ? __dmul_rn(p.hscale, p.hv[x]) : p.hv[x]);
-                store_val(dst + x, m);
-                if (p.amin) p.amin[x] = p.dhi - t;
-                edges += on_edge(t, p.weff);
-            }
-        }
+        edges = write_rows_strided<T, OFF>(p, tl, su, tt, kr64);
     }
     count_edges(p, edges);
 }
@@ -1031,18 +1120,8 @@ struct BatchItem {
     int use_tma, pad;
 };
 
-// One axis pass over many grids of the same launch shape: block b handles
-// tile (b mod tiles) of instance (b / tiles).  Fields that differ between
-// instances come from `items`; the rest of `p` is shared.
-template <typename T, int LAYOUT, int ALGO>
-__global__ void __launch_bounds__(1024) pass_kernel_batch(const BatchItem *__restrict__ items, PassParams p,
-                                                          long long count)
+__device__ __forceinline__ void batch_fields(PassParams &q, const BatchItem *it)
 {
-    const long long inst = blockIdx.x / p.ntiles;
-    const long long tile = blockIdx.x - inst * p.ntiles;
-    if (inst >= count) return;
-    const BatchItem *it = items + inst;
-    PassParams q = p;
     q.src = it->src;
     q.dst = it->dst;
     q.hv = it->hv;
@@ -1052,6 +1131,21 @@ __global__ void __launch_bounds__(1024) pass_kernel_batch(const BatchItem *__res
     q.hoff = it->hoff;
     q.dhi = it->dhi;
     q.use_tma = it->use_tma;
+}
+
+// One axis pass over many grids of the same launch shape: block b handles
+// tile (b mod tiles) of instance (b / tiles).  Fields that differ between
+// instances come from `items`; the rest of `p` is shared.
+template <typename T, int LAYOUT, int ALGO>
+__global__ void __launch_bounds__(1024) pass_kernel_batch(const BatchItem *__restrict__ items, PassParams p,
+                                                          long long count)
+{
+    const unsigned inst = blockIdx.x / (unsigned)p.ntiles;
+    const long long tile = blockIdx.x - inst * (unsigned)p.ntiles;
+    if (inst >= count) return;
+    const BatchItem *it = items + inst;
+    PassParams q = p;
+    batch_fields(q, it);
     if (q.use_tma && LAYOUT == LAYOUT_STRIDED && threadIdx.x == 0)
         asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(&it->tmap) : "memory");
     pass_tile<T, LAYOUT, ALGO>(&it->tmap, q, tile);

@@ -11,6 +11,7 @@
 
 #include "hjlo.h"
 #include "hjlo_device.cuh"
+#include "hjlo_dense.cuh"
 #include "hjlo_persist.cuh"
 
 namespace hjlo {
@@ -32,6 +33,8 @@ struct AxisPlan {
     int wide_mul = 2, wide_add = 8;        // warp offload of wide brackets (see PassParams)
     int t8_ok = 1;                         // MONGE: argmin offsets may be bytes (single-grid launches)
     int t8 = 0;                            // MONGE: argmin offsets are bytes (weff <= 256 and t8_ok)
+    int dense = 0;                         // MONGE: rows per segment of the banded search (0: divide and conquer)
+    int off_kp = 0, off_q = 0, qcap = 0;   // banded search: see PassParams
     double eta = 0.0;                      // DECOMP: convexity tolerance of the decomposition
     // DECOMP with a period cut across CTAs (dsplit = 1): chunks of dchunk
     // points (dB per line) for the cut, write-back blocks of dvR outputs
@@ -101,6 +104,9 @@ hjlo_status shape_launch(AxisPlan &ax, int esize, int algo, int num_sms, size_t 
 // Candidate shapes around ax's current one for the autotuner: lanes per line
 // and lines per tile halved / kept / doubled, offload on / off.
 std::vector<ShapeHints> tune_candidates(const AxisPlan &ax);
+
+// Whether a bulk copy per tile can stage contiguous lines of `ptr`.
+bool contig_tma(const AxisPlan &ax, int esize, const void *ptr);
 
 // 3D TMA descriptor {inner, N, outer} of `ptr` for lines along a strided
 // axis; false if TMA cannot serve this pointer/shape.

@@ -144,9 +144,33 @@ hjlo_status resolve_axis(long long N, double dx, double h, double P, long long W
 
 static size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
+// Halo pitch: at least N + weff - 1 words; when several lines share a warp
+// (lpl < 32) the pitch is congruent to lpl*seg mod 32, so that lane g of line
+// l reads bank S*(lpl*l + g) mod 32 -- distinct across the warp.
+static int halo_pitch(const AxisPlan &ax)
+{
+    // the banded search reads past the halo, in full bands
+    long long L = ax.N + ax.weff - 1 + (ax.dense ? kDenseOver : 0);
+    if (ax.lpl >= 32) {
+        // a warp writes the keys of 32 / C positions of C strided lines: lines
+        // 32 / C banks apart keep them apart
+        if (ax.dense && ax.layout == LAYOUT_STRIDED)
+            while (L % 32 != std::max(32 / ax.C, ax.dense == kFlat ? 4 : 1) % 32) ++L;
+        return (int)align_up((size_t)L, ax.dense && ax.dense != kFlat ? 1 : 4);
+    }
+    if (ax.dense == kFlat) {                     // 16-byte rows of keys, lines a few banks apart
+        while (L % 32 != std::max(32 / ax.C, 4) % 32) ++L;
+        return (int)L;
+    }
+    long long want = ((long long)ax.lpl * ax.seg) % 32;
+    while (L % 32 != want) ++L;
+    return (int)L;
+}
+
 static void layout_smem(AxisPlan &ax, int esize, int algo)
 {
     const int C = ax.C;
+    if (ax.dense) ax.lp = halo_pitch(ax);                    // depends on C
     const long long rows = (ax.layout == LAYOUT_STRIDED) ? (long long)ax.nbox * ax.by : ax.N;
     const bool monge = (algo == KALGO_MONGE);
     size_t off = 0;
@@ -155,13 +179,25 @@ static void layout_smem(AxisPlan &ax, int esize, int algo)
     ax.off_fx = (int)off;
     if (monge) off = align_up(off + (size_t)C * ax.lp * 4, 16);
     ax.off_kfx = (int)off;
-    if (monge) off = align_up(off + (size_t)C * ax.weff * 4, 16);
+    if (monge && !ax.dense) off = align_up(off + (size_t)C * ax.weff * 4, 16);
+    if (ax.dense) {
+        // one table per tile, a copy with chunk numbers, per group of lanes a
+        // queue of flagged rows (an eighth of its rows; when it runs over,
+        // every row is looked at)
+        const int group = std::max(32, ax.lpl), groups = std::max(1, C * ax.lpl / group);
+        off = align_up(off + (size_t)(kDenseLow + ax.weff + kDenseHigh) * 4, 16);
+        ax.off_kp = (int)off;
+        off = align_up(off + (size_t)((ax.weff + 3) & ~3) * 4, 16);
+        ax.off_q = (int)off;
+        ax.qcap = std::max(31, (int)(group / ax.lpl * ax.N / 8));
+        off = align_up(off + (size_t)groups * (ax.qcap + 1) * 4, 16);
+    }
     ax.off_t = (int)off;
     off = align_up(off + (size_t)C * ax.tp * (ax.t8 ? 1 : 2), 16);
     ax.off_k64 = (int)off;
     off = align_up(off + (size_t)ax.weff * 8, 16);
     ax.off_misc = (int)off;
-    off = align_up(off + 16 + 40 * (size_t)C, 16);   // mbarrier, counters, per-line screen facts
+    off = align_up(off + 16 + 40 * (size_t)C, 16);   // mbarrier, screen facts
     ax.smem = off;
 }
 
@@ -178,18 +214,6 @@ static int ilog2(int x)
     return r;
 }
 
-// Halo pitch: at least N + weff - 1 words; when several lines share a warp
-// (lpl < 32) the pitch is congruent to lpl*seg mod 32, so that lane g of line
-// l reads bank S*(lpl*l + g) mod 32 -- distinct across the warp.
-static int halo_pitch(const AxisPlan &ax)
-{
-    long long L = ax.N + ax.weff - 1;
-    if (ax.lpl >= 32) return (int)align_up((size_t)L, 4);
-    long long want = ((long long)ax.lpl * ax.seg) % 32;
-    while (L % 32 != want) ++L;
-    return (int)L;
-}
-
 // Pivot group size: GS lanes share one whole-window scan (weff/GS candidates
 // each) and the other GS-1 first rows are bracketed by group pivots (about
 // GS*S candidates).  Returns the group size and its cost in candidates per lane.
@@ -203,6 +227,50 @@ static int pivot_group(int weff, int S, int lpl, double *cost)
     }
     if (cost) *cost = bc;
     return best;
+}
+
+// The banded search's kind (rows per segment; hjlo_dense.cuh) and its lanes per
+// line, or 0 for divide and conquer.  `cmin`: the fewest lines a tile can hold.
+// Flat for windows of up to kFlatMaxWindow: the fewest lanes a line that give
+// every SM 512 threads and a lane four turns of four rows at most, since the
+// more lines a tile then holds, the longer its rows in memory (256^3 grid,
+// strided axes: tiles of 4, 8, 16 lines 229, 175, 157 us a pass); more lanes
+// where that leaves fewer of them idle.  Above that window (129 displacements
+// on the 1024^2 grid: flat 31 us, bands 27), one lane holds a segment's rows but
+// the first in registers, 9 or 13 rows a segment; a power of two of lanes then
+// leaves at most 30 % of them idle, and a pivot scans the whole window, weff / 9
+// add-minimums and shared-memory words a row, which bounds the windows.
+static int dense_segment(const AxisPlan &ax, long long NR, long long nlines, int cmin, int num_sms,
+                         const ShapeHints &hint, int *lanes)
+{
+    if (ax.weff > kDenseMaxWindow) return 0;
+    const bool hinted = hint.lpl > 0 && (hint.lpl & (hint.lpl - 1)) == 0 && hint.lpl <= ax.N;
+    if (ax.weff <= kFlatMaxWindow) {
+        const long long quads = (NR + 3) / 4;
+        const int most = dense_threads(kFlat) / cmin;
+        int best = 1;
+        double score = 0.0;
+        for (int lpl = 1; lpl <= most && lpl <= ax.N; lpl *= 2) {
+            const long long turns = (quads + lpl - 1) / lpl;
+            if (2 * lpl <= most && turns > 1 && (turns > 4 || nlines * lpl < 512LL * num_sms)) continue;
+            const double use = (double)quads / (double)(turns * lpl);
+            if (use > 1.1 * score) { score = use; best = lpl; }
+        }
+        if (hinted && hint.lpl <= most) best = hint.lpl;
+        *lanes = best;
+        return (quads + best - 1) / best <= 16 ? kFlat : 0;
+    }
+    int lpl = 1;
+    while (13LL * lpl < NR) lpl *= 2;
+    if (hinted) lpl = hint.lpl;
+    const long long rows = (NR + lpl - 1) / lpl;
+    if (rows > 13 || (long long)lpl * cmin > dense_threads(13)) return 0;
+    // few lanes in all: a pivot's scan of the window, done by one lane, would be
+    // most of the launch (8192-point line, 291 displacements, 15 blocks: 15 us
+    // a pass against 11.7 by divide and conquer, which shares it)
+    if (!hinted && nlines * lpl < 64LL * num_sms) return 0;
+    *lanes = lpl;
+    return rows <= 9 && lpl * cmin <= dense_threads(9) ? 9 : 13;
 }
 
 ShapeHints env_hints()
@@ -363,7 +431,20 @@ static hjlo_status shape_lines(AxisPlan &ax, int esize, int algo, int num_sms, s
 
     // rows searched per line (a row block searches only its own rows)
     const long long NR = (ax.rows > 0 && ax.rows < N) ? ax.rows : N;
-    if (algo == KALGO_MONGE) {
+    ax.dense = (algo == KALGO_MONGE) ? dense_segment(ax, NR, nlines, cmin, num_sms, hint, &ax.lpl) : 0;
+    if (ax.dense) {
+        ax.log2lpl = ilog2(ax.lpl);
+        ax.seg = odd_at_least((NR + ax.lpl - 1) / ax.lpl);
+        if (ax.dense != kFlat) ax.seg = ax.dense;
+        ax.gs = 1;
+        ax.t8 = 0;
+        ax.tp = (int)N;
+        while (ax.tp % 4 != 2) ++ax.tp;
+        ax.wide_mul = 2;
+        ax.wide_add = 8;
+        ax.lp = halo_pitch(ax);
+        ax.wpl = 1;
+    } else if (algo == KALGO_MONGE) {
         // lanes per line: maximise (occupancy efficiency) / (work per row), with
         // work per row ~ weff/S + log2(S) + 3 (pivot share, divide and conquer,
         // staging and write-back) and occupancy bounded by shared memory per
@@ -431,10 +512,11 @@ static hjlo_status shape_lines(AxisPlan &ax, int esize, int algo, int num_sms, s
     };
     ax.C = C;
     layout_smem(ax, esize, algo);
-    if (ax.smem > smem_optin || (long long)C * lanes > 1024)
+    const long long most = ax.dense ? dense_threads(ax.dense) : 1024;
+    if (ax.smem > smem_optin || (long long)C * lanes > most)
         return set_error(HJLO_EUNSUPPORTED, "a line of %lld points does not fit in shared memory", N);
     const size_t budget = std::min<size_t>(110 * 1024, smem_optin);
-    const long long cap = (algo == KALGO_MONGE) ? 128 : 512;
+    const long long cap = (algo == KALGO_MONGE) ? (ax.dense ? 256 : 128) : 512;
     while (2 * C <= std::max(cmax, C) && (long long)2 * C * lanes <= cap &&
            tiles_for(2 * C) * std::max(1LL, replicas) >= 2LL * num_sms) {
         AxisPlan t = ax;
@@ -446,7 +528,8 @@ static hjlo_status shape_lines(AxisPlan &ax, int esize, int algo, int num_sms, s
     // hinted lines per tile (a power of two that fits)
     if (hint.C > 0) {
         const int want = hint.C;
-        if (want >= cmin && (want & (want - 1)) == 0 && (long long)want * lanes <= 1024) {
+        if (want >= cmin && (want & (want - 1)) == 0 && (long long)want * lanes <= most &&
+            (!ax.dense || want * lanes >= 32)) {
             AxisPlan t = ax;
             t.C = want;
             layout_smem(t, esize, algo);
@@ -477,6 +560,13 @@ static PFN_cuTensorMapEncodeTiled_v12000 encode_fn()
             fn = (PFN_cuTensorMapEncodeTiled_v12000)p;
     });
     return fn;
+}
+
+// Lines along the contiguous axis are staged by one bulk copy per tile: whole
+// lines, tiles that start on 16-byte boundaries.
+bool contig_tma(const AxisPlan &ax, int esize, const void *ptr)
+{
+    return ax.vblocks == 1 && ((uintptr_t)ptr & 15) == 0 && ((ax.N * ax.C * esize) & 15) == 0;
 }
 
 // 3D view {inner, N, outer} of the grid for lines along a strided axis; box
@@ -575,6 +665,10 @@ void fill_params(const AxisPlan &ax, PassParams &p)
     p.off_t = ax.off_t;
     p.off_k64 = ax.off_k64;
     p.off_misc = ax.off_misc;
+    p.off_kp = ax.off_kp;
+    p.off_q = ax.off_q;
+    p.qcap = ax.qcap;
+    p.dense = ax.dense;
     p.wait_ns = ax.wait_ns;    // 0.5 s unless a test shortens it: a tile copy takes microseconds
     p.test_extra_tx = ax.test_extra_tx;
     p.wide_mul = ax.wide_mul;
@@ -645,7 +739,7 @@ hjlo_status launch_pass(const AxisPlan &ax, int dtype, const void *src, void *ds
     CUtensorMap map;
     memset(&map, 0, sizeof(map));
     if (ax.layout == LAYOUT_CONTIG) {
-        p.use_tma = (ax.vblocks == 1) && (((uintptr_t)src & 15) == 0) && (((ax.N * esize) & 15) == 0);
+        p.use_tma = contig_tma(ax, esize, src) ? 1 : 0;
     } else {
         p.use_tma = encode_strided(ax, esize, src, &map) ? 1 : 0;
     }

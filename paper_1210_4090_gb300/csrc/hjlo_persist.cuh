@@ -2,7 +2,7 @@
 // step of every instance of a batch in one launch (see pass_kernel_persist).
 #pragma once
 
-#include "hjlo_device.cuh"
+#include "hjlo_dense.cuh"
 
 namespace hjlo {
 
@@ -39,6 +39,20 @@ struct PersistParams {
 __device__ __forceinline__ void mbar_inval(uint64_t *bar)
 {
     asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_addr(bar)) : "memory");
+}
+
+// One tile by the search its shape was made for.
+template <typename T, int LAYOUT>
+__device__ __forceinline__ void persist_tile(const CUtensorMap *tmap, const PassParams &p, long long tile)
+{
+    if (p.dense == kFlat)
+        dense_tile<T, LAYOUT, unsigned short, kFlat>(tmap, p, tile);
+    else if (p.dense == 9)
+        dense_tile<T, LAYOUT, unsigned short, 9>(tmap, p, tile);
+    else if (p.dense == 13)
+        dense_tile<T, LAYOUT, unsigned short, 13>(tmap, p, tile);
+    else
+        pass_tile<T, LAYOUT, KALGO_MONGE>(tmap, p, tile);
 }
 
 // All passes of one time step of every instance in one launch: CTAs take
@@ -119,9 +133,9 @@ __global__ void __launch_bounds__(1024) pass_kernel_persist(const __grid_constan
             const bool contig = (s_p.inner == 1);
             for (int t = 0; t < it.ntile; ++t) {
                 if (contig)
-                    pass_tile<T, LAYOUT_CONTIG, KALGO_MONGE>(&bi->tmap, s_p, it.tile0 + t);
+                    persist_tile<T, LAYOUT_CONTIG>(&bi->tmap, s_p, it.tile0 + t);
                 else
-                    pass_tile<T, LAYOUT_STRIDED, KALGO_MONGE>(&bi->tmap, s_p, it.tile0 + t);
+                    persist_tile<T, LAYOUT_STRIDED>(&bi->tmap, s_p, it.tile0 + t);
                 __syncthreads();
                 if (tid == 0) mbar_inval(reinterpret_cast<uint64_t *>(pass_smem() + s_p.off_misc));
                 __syncthreads();

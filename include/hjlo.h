@@ -387,7 +387,10 @@ hjlo_status hjlo_sync(hjlo_plan *plan, hjlo_counters *out);
  * copied.  desc->dtype must be HJLO_F64, desc->algo AUTO or BRUTE.  Tables
  * (per point and mode, per displacement) are formed on the host in binary64
  * with the C library's sin and cos; the sum over modes uses fused
- * multiply-adds.  Errors: HJLO_EINVAL, HJLO_EUNSUPPORTED
+ * multiply-adds.  The path integrals of all sources and displacements are
+ * kept on the device (grid x box binary64 values) where that is at most 1 GiB
+ * and can be allocated; steps sum them anew otherwise, with the same results.
+ * Errors: HJLO_EINVAL, HJLO_EUNSUPPORTED
  * (grid x box x modes too large), HJLO_ENOMEM, HJLO_ECUDA.
  */
 typedef struct hjlo_integral hjlo_integral;

@@ -16,11 +16,19 @@
 //
 // Tables are formed once per plan on the host (libm sin / cos): A per point
 // and mode (mode-major, so the threads of a warp read consecutive sources),
-// K and phi per displacement.  Four threads per output point (consecutive
-// lanes) share its displacements and merge their minima by shuffles;
-// ping-pong buffers (a step reads its whole source before any output is
+// K and phi per displacement.  h * S depends on neither u nor the step, so the
+// plan also holds it for every source and displacement (8 bytes a candidate,
+// up to kCostBytes): a step then is one load, an add and a subtract a
+// candidate instead of 4 fused multiply-adds a mode as well.  128^2 grid, 81
+// displacements, 12 modes: 92 us a step (binary64 pipe 73 % busy) without the
+// table, 10.5 with it, where two binary64 operations a candidate are 5.
+// Larger boxes sum S in the step, four threads per output point (consecutive
+// lanes) sharing its displacements and merging their minima by shuffles.
+// Ping-pong buffers (a step reads its whole source before any output is
 // final).
+#include <algorithm>
 #include <cmath>
+#include <cstdlib>
 #include <cstring>
 #include <new>
 #include <vector>
@@ -42,12 +50,40 @@ struct hjlo_integral {
     double *d_phi = nullptr;      // [ndisp][nmodes][2]
     int *d_disp = nullptr;        // [ndisp][3] displacement per axis, mod N
     double *d_tmp = nullptr;      // ping-pong buffer, npts
+    double *d_hS = nullptr;       // [ndisp][npts]: h S(y, d), or null
     long long steps = 0;
 };
 
 namespace {
 
 constexpr int kIntegralSplit = 4;      // threads per output point
+
+// key2 with NaN above everything.
+using dkey_pair = Key2;
+__device__ __forceinline__ dkey_pair dkey_of(double x)
+{
+    const unsigned hi = (unsigned)__double2hiint(x) & 0x7fffffffu, lo = (unsigned)__double2loint(x);
+    return (hi > 0x7ff00000u || (hi == 0x7ff00000u && lo)) ? key2_max() : key2(x);
+}
+
+// S(y, d) of one source and displacement, in the fixed order.
+__device__ __forceinline__ double path_sum(const double *__restrict__ A, const double *__restrict__ ph, long long y,
+                                           int nmodes, long long npts)
+{
+    double se = 0.0, so = 0.0;
+    int m = 0;
+    for (; m + 1 < nmodes; m += 2) {
+        se = __fma_rn(A[(long long)m * npts + y], ph[2 * m], se);
+        se = __fma_rn(-A[((long long)nmodes + m) * npts + y], ph[2 * m + 1], se);
+        so = __fma_rn(A[(long long)(m + 1) * npts + y], ph[2 * m + 2], so);
+        so = __fma_rn(-A[((long long)nmodes + m + 1) * npts + y], ph[2 * m + 3], so);
+    }
+    if (m < nmodes) {
+        se = __fma_rn(A[(long long)m * npts + y], ph[2 * m], se);
+        se = __fma_rn(-A[((long long)nmodes + m) * npts + y], ph[2 * m + 1], se);
+    }
+    return __dadd_rn(se, so);
+}
 
 __global__ void integral_kernel(const double *__restrict__ src, double *__restrict__ dst,
                                 const double *__restrict__ A, const double *__restrict__ K,
@@ -73,19 +109,7 @@ __global__ void integral_kernel(const double *__restrict__ src, double *__restri
             y2 += (y2 < 0) ? m2 : 0;
             const long long y = ((long long)y0 * m1 + y1) * m2 + y2;
             const double *ph = phi + 2 * (long long)nmodes * di;
-            double se = 0.0, so = 0.0;
-            int m = 0;
-            for (; m + 1 < nmodes; m += 2) {
-                se = __fma_rn(A[(long long)m * npts + y], ph[2 * m], se);
-                se = __fma_rn(-A[((long long)nmodes + m) * npts + y], ph[2 * m + 1], se);
-                so = __fma_rn(A[(long long)(m + 1) * npts + y], ph[2 * m + 2], so);
-                so = __fma_rn(-A[((long long)nmodes + m + 1) * npts + y], ph[2 * m + 3], so);
-            }
-            if (m < nmodes) {
-                se = __fma_rn(A[(long long)m * npts + y], ph[2 * m], se);
-                se = __fma_rn(-A[((long long)nmodes + m) * npts + y], ph[2 * m + 1], se);
-            }
-            const double S = __dadd_rn(se, so);
+            const double S = path_sum(A, ph, y, nmodes, npts);
             const double c = __dsub_rn(__dadd_rn(src[y], K[di]), __dmul_rn(h, S));
             best = (c < best) ? c : best;
         }
@@ -98,6 +122,71 @@ __global__ void integral_kernel(const double *__restrict__ src, double *__restri
     if (live && part == 0) dst[x] = best;
 }
 
+constexpr size_t kCostBytes = size_t(1) << 30;     // table of h S: at most this much
+
+__global__ void integral_cost_kernel(double *__restrict__ hS, const double *__restrict__ A,
+                                     const double *__restrict__ phi, long long ndisp, int nmodes, long long npts,
+                                     double h)
+{
+    const long long n = ndisp * npts;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        const long long di = i / npts, y = i - di * npts;
+        hS[i] = __dmul_rn(h, path_sum(A, phi + 2 * (long long)nmodes * di, y, nmodes, npts));
+    }
+}
+
+constexpr int kCostParts = 8;          // warps that share 32 outputs
+
+// One step from the table: a warp's lanes hold consecutive outputs (the table's
+// rows are read whole), a block's warps share the displacements.  Candidates are
+// compared as order-preserving 32-bit pairs, which leaves the binary64 pipe to
+// the add and the subtract; a NaN never wins, as with a binary64 comparison.
+__global__ void __launch_bounds__(32 * kCostParts) integral_table_kernel(
+    const double *__restrict__ src, double *__restrict__ dst, const double *__restrict__ hS,
+    const double *__restrict__ K, const int *__restrict__ disp, int ndisp, int n0, int n1, int n2, long long npts)
+{
+    __shared__ double part[kCostParts][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const long long x = blockIdx.x * 32LL + lane;
+    double best = INFINITY;
+    if (x < npts) {
+        const unsigned xu = (unsigned)x;                       // npts <= 2^31
+        const unsigned r = xu / (unsigned)n2;
+        const int i2 = (int)(xu - r * (unsigned)n2), i0 = (int)(r / (unsigned)n1), i1 = (int)(r - (unsigned)i0 * n1);
+        dkey_pair bk = dkey_of(best);
+#pragma unroll 4
+        for (int di = warp; di < ndisp; di += kCostParts) {
+            // displacements are stored mod N: one conditional add wraps
+            int y0 = i0 - __ldg(disp + 3 * di), y1 = i1 - __ldg(disp + 3 * di + 1), y2 = i2 - __ldg(disp + 3 * di + 2);
+            y0 += (y0 < 0) ? n0 : 0;
+            y1 += (y1 < 0) ? n1 : 0;
+            y2 += (y2 < 0) ? n2 : 0;
+            const long long y = ((long long)y0 * n1 + y1) * n2 + y2;
+            const double c = __dsub_rn(__dadd_rn(src[y], __ldg(K + di)), __ldg(hS + di * npts + y));
+            const dkey_pair ck = dkey_of(c);
+            if (key2_less(ck, bk)) {
+                bk = ck;
+                best = c;
+            }
+        }
+    }
+    part[warp][lane] = best;
+    __syncthreads();
+    if (warp == 0 && x < npts) {
+        dkey_pair bk = dkey_of(best);
+#pragma unroll
+        for (int w = 1; w < kCostParts; ++w) {
+            const double c = part[w][lane];
+            const dkey_pair ck = dkey_of(c);
+            if (key2_less(ck, bk)) {
+                bk = ck;
+                best = c;
+            }
+        }
+        dst[x] = best;
+    }
+}
+
 void release(hjlo_integral *s)
 {
     cudaFree(s->d_A);
@@ -105,6 +194,7 @@ void release(hjlo_integral *s)
     cudaFree(s->d_phi);
     cudaFree(s->d_disp);
     cudaFree(s->d_tmp);
+    cudaFree(s->d_hS);
 }
 
 }  // namespace
@@ -228,6 +318,27 @@ hjlo_status hjlo_integral_create(const hjlo_desc *d, int32_t nmodes, const int32
         delete s;
         return st;
     }
+    // the table of h S, where it fits: without it a step sums S itself
+    // (HJLO_TEST_COST_BYTES: a test's limit)
+    const size_t bytes = sizeof(double) * (size_t)s->npts * (size_t)s->ndisp;
+    const char *env = getenv("HJLO_TEST_COST_BYTES");
+    if (nmodes > 0 && bytes <= (env ? (size_t)std::max(0LL, atoll(env)) : kCostBytes)) {
+        if (cudaMalloc(&s->d_hS, bytes) == cudaSuccess) {
+            const long long blocks = std::min<long long>((s->npts * s->ndisp + 255) / 256, 1 << 20);
+            integral_cost_kernel<<<(unsigned)blocks, 256, 0, s->stream>>>(s->d_hS, s->d_A, s->d_phi, s->ndisp, nmodes,
+                                                                          s->npts, s->h);
+            cudaError_t e = cudaGetLastError();
+            if (e != cudaSuccess) {
+                st = cuda_error(e, "integral cost kernel launch");
+                release(s);
+                delete s;
+                return st;
+            }
+        } else {
+            s->d_hS = nullptr;
+            cudaGetLastError();
+        }
+    }
     *out = s;
     return HJLO_OK;
 }
@@ -242,8 +353,13 @@ hjlo_status hjlo_integral_run(hjlo_integral *s, double *u, int64_t nsteps)
     double *a = u, *b = s->d_tmp;
     const unsigned blocks = (unsigned)((s->npts * kIntegralSplit + 255) / 256);
     for (long long n = 0; n < nsteps; ++n) {
-        integral_kernel<<<blocks, 256, 0, s->stream>>>(a, b, s->d_A, s->d_K, s->d_phi, s->d_disp, s->ndisp, s->nmodes,
-                                                       s->shape[0], s->shape[1], s->shape[2], s->npts, s->h);
+        if (s->d_hS)
+            integral_table_kernel<<<(unsigned)((s->npts + 31) / 32), 32 * kCostParts, 0, s->stream>>>(
+                a, b, s->d_hS, s->d_K, s->d_disp, (int)s->ndisp, (int)s->shape[0], (int)s->shape[1], (int)s->shape[2],
+                s->npts);
+        else
+            integral_kernel<<<blocks, 256, 0, s->stream>>>(a, b, s->d_A, s->d_K, s->d_phi, s->d_disp, s->ndisp, s->nmodes,
+                                                           s->shape[0], s->shape[1], s->shape[2], s->npts, s->h);
         e = cudaGetLastError();
         if (e != cudaSuccess) return cuda_error(e, "integral kernel launch");
         std::swap(a, b);

@@ -89,6 +89,7 @@ __global__ void __launch_bounds__(256) adjoint_pass_kernel(AdjParams p)
     adj_tile<LAYOUT>(p, blockIdx.x, base, lstride, pstride, valid, line0, linestep);
 
     if (tid < C) mono[tid] = 1;
+    pdl_wait();
     for (int idx = tid; idx < C * N; idx += nthr) {
         int l, i;
         if (LAYOUT == LAYOUT_CONTIG) { l = idx / N; i = idx - l * N; }
@@ -123,6 +124,7 @@ __global__ void __launch_bounds__(256) adjoint_pass_kernel(AdjParams p)
             for (int L = la[N - 1] + 1; L <= a0 + N + 1; ++L) lf[L - a0] = N;
     }
     __syncthreads();
+    pdl_next();
     // gather, ascending target order
     for (int idx = tid; idx < C * N; idx += nthr) {
         int l, r;
@@ -286,11 +288,9 @@ hjlo_status launch_adjoint_pass(const AxisPlan &ax, double dx, double *ub, const
     p.C = sh.C;
     p.log2C = sh.log2C;
     p.dx = dx;
-    if (sh.layout == LAYOUT_CONTIG)
-        adjoint_pass_kernel<LAYOUT_CONTIG><<<(unsigned)sh.ntiles, sh.threads, sh.smem, st>>>(p);
-    else
-        adjoint_pass_kernel<LAYOUT_STRIDED><<<(unsigned)sh.ntiles, sh.threads, sh.smem, st>>>(p);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_pdl(sh.layout == LAYOUT_CONTIG ? adjoint_pass_kernel<LAYOUT_CONTIG>
+                                                          : adjoint_pass_kernel<LAYOUT_STRIDED>,
+                               (unsigned)sh.ntiles, sh.threads, sh.smem, st, p);
     if (e != cudaSuccess) return cuda_error(e, "adjoint pass launch");
     return HJLO_OK;
 }

@@ -450,12 +450,9 @@ hjlo_status hjlo_step(hjlo_plan *p, const void *u_in, void *u_out, const double 
     if (u_in != u_out && ranges_overlap(u_in, u_out, bytes))
         return set_error(HJLO_EINVAL, "u_in and u_out overlap without being equal");
     if ((s = set_device(p)) != HJLO_OK) return s;
-    const double *hv = nullptr;
-    if (V) {
-        if ((s = form_hv(p, V)) != HJLO_OK) return s;
-        hv = p->d_hv;
-    }
-    s = enqueue_step(p, u_in, u_out, hv, 0.0, argmin_out, p->stream);
+    // the last pass forms fl(h V) itself: one launch and a grid's traffic less
+    // than a table of it, which pays for itself in runs of several steps
+    s = enqueue_step(p, u_in, u_out, V, V ? p->desc.h : 0.0, argmin_out, p->stream);
     if (s == HJLO_OK) p->steps += 1;
     return s;
 }

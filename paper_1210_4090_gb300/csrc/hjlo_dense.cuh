@@ -708,6 +708,7 @@ __device__ __forceinline__ void dense_tile(const CUtensorMap *tmap, const PassPa
         if (lane == 0 && wr) atomicAdd(&p.counters[CNT_RESCAN], (unsigned long long)wr);
     }
     // ---- exact values, potential term, stores
+    pdl_next();
     int edges = 0;
     if constexpr (LAYOUT == LAYOUT_CONTIG) {
         if (cl < tl.valid) {

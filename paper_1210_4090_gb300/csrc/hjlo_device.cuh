@@ -186,6 +186,13 @@ __device__ __forceinline__ void tma_tensor_load_3d(void *dst, const CUtensorMap 
         : "memory");
 }
 
+// Programmatic dependent launch: the next pass's CTAs may come up, and set up,
+// once every CTA of this one is at its write-back (earlier, they would gather on
+// the SMs that happen to have room); before a CTA touches what the passes
+// before it wrote (or writes what they read), it waits for them to end.
+__device__ __forceinline__ void pdl_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Hint: bring [p, p + bytes) of global memory into L2 ahead of use (whole
 // 16-byte units inside the range only; the ragged ends load normally).
 __device__ __forceinline__ void prefetch_l2(const void *p, unsigned long long bytes)
@@ -729,9 +736,10 @@ __device__ __forceinline__ bool stage_tile(const CUtensorMap *tmap, const PassPa
         mbar_init(bar, 1);
         fence_mbar_init();
     }
-    __syncthreads();
-    stage_issue<T, LAYOUT>(tmap, p, tile, su, bar);
     for (int i = threadIdx.x; i < p.weff; i += blockDim.x) copy_async(kr64 + i, p.kr64 + i);
+    __syncthreads();
+    pdl_wait();
+    stage_issue<T, LAYOUT>(tmap, p, tile, su, bar);
     return stage_wait(p, bar, 0);
 }
 
@@ -1023,6 +1031,7 @@ __device__ __forceinline__ void pass_tile(const CUtensorMap *tmap, const PassPar
             // stay inside the warp after P2), so each warp writes its own rows
             // back as soon as it is done: no block barrier, coalesced stores.
             __syncwarp();
+            pdl_next();
             const int nl = (lpl >= 32) ? 1 : (32 >> p.log2lpl);     // lines held by this warp
             int edges = 0;
             for (int k = 0; k < nl; ++k) {
@@ -1080,6 +1089,7 @@ __device__ __forceinline__ void pass_tile(const CUtensorMap *tmap, const PassPar
     __syncthreads();
 
     // ---- exact values, potential term, stores (coalesced order)
+    pdl_next();
     int edges = 0;
     if constexpr (LAYOUT == LAYOUT_CONTIG) {
         const int lanes = nthr >> p.log2C;              // threads per line

@@ -21,7 +21,7 @@
 // up to kCostBytes): a step then is one load, an add and a subtract a
 // candidate instead of 4 fused multiply-adds a mode as well.  128^2 grid, 81
 // displacements, 12 modes: 92 us a step (binary64 pipe 73 % busy) without the
-// table, 10.5 with it, where two binary64 operations a candidate are 5.
+// table, 8.7 with it, where two binary64 operations a candidate are 5.
 // Larger boxes sum S in the step, four threads per output point (consecutive
 // lanes) sharing its displacements and merging their minima by shuffles.
 // Ping-pong buffers (a step reads its whole source before any output is
@@ -146,6 +146,7 @@ __global__ void __launch_bounds__(32 * kCostParts) integral_table_kernel(
     const double *__restrict__ K, const int *__restrict__ disp, int ndisp, int n0, int n1, int n2, long long npts)
 {
     __shared__ double part[kCostParts][32];
+    pdl_wait();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long x = blockIdx.x * 32LL + lane;
     double best = INFINITY;
@@ -171,6 +172,7 @@ __global__ void __launch_bounds__(32 * kCostParts) integral_table_kernel(
         }
     }
     part[warp][lane] = best;
+    pdl_next();
     __syncthreads();
     if (warp == 0 && x < npts) {
         dkey_pair bk = dkey_of(best);
@@ -354,13 +356,13 @@ hjlo_status hjlo_integral_run(hjlo_integral *s, double *u, int64_t nsteps)
     const unsigned blocks = (unsigned)((s->npts * kIntegralSplit + 255) / 256);
     for (long long n = 0; n < nsteps; ++n) {
         if (s->d_hS)
-            integral_table_kernel<<<(unsigned)((s->npts + 31) / 32), 32 * kCostParts, 0, s->stream>>>(
-                a, b, s->d_hS, s->d_K, s->d_disp, (int)s->ndisp, (int)s->shape[0], (int)s->shape[1], (int)s->shape[2],
-                s->npts);
+            e = launch_pdl(integral_table_kernel, (unsigned)((s->npts + 31) / 32), 32 * kCostParts, 0, s->stream, a, b,
+                           s->d_hS, s->d_K, s->d_disp, (int)s->ndisp, (int)s->shape[0], (int)s->shape[1],
+                           (int)s->shape[2], s->npts);
         else
             integral_kernel<<<blocks, 256, 0, s->stream>>>(a, b, s->d_A, s->d_K, s->d_phi, s->d_disp, s->ndisp, s->nmodes,
                                                            s->shape[0], s->shape[1], s->shape[2], s->npts, s->h);
-        e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaGetLastError();
         if (e != cudaSuccess) return cuda_error(e, "integral kernel launch");
         std::swap(a, b);
     }

@@ -55,6 +55,27 @@ struct AxisPlan {
     int off_u = 0, off_fx = 0, off_kfx = 0, off_t = 0, off_k64 = 0, off_misc = 0;
 };
 
+// Launches a kernel that waits for its predecessors itself (pdl_wait), so that
+// it may start before they end: 1-2 us of each launch of a chain of small ones
+// (gradients on 512^2, 128 steps: 8.8 -> 7.7 ms; 8192-point line, 289 steps:
+// 3.3 -> 2.6).  Of the larger grids 90x121x135 gains 10 %, 256^3 2 %, and
+// 701 x 1013 loses 6 %.
+template <typename... P, typename... A>
+cudaError_t launch_pdl(void (*kernel)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t st, A &&...args)
+{
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // Records an error for hjlo_last_error() and returns it.
 hjlo_status set_error(hjlo_status st, const char *fmt, ...);
 hjlo_status cuda_error(cudaError_t e, const char *what);

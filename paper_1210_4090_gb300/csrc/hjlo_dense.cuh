@@ -29,7 +29,10 @@
 // 4 (S - 1) add-minimums.  Segments with more than 16 sources (shocks) are
 // shared by the lanes of the warp, two rows a lane, several lanes a source
 // range when few segments are left.  1024^2 grid, 129 displacements: 27 -> 19
-// us a pass.
+// us a pass.  Above kScanWindow displacements (kWide) the lanes of a warp find
+// the pivots together, halving the distance between known ones; four number
+// bits leave room for the curvature of a window that wide (its square over 2^23
+// of the table's range), up to kDenseMaxWindow.
 //
 // Making it exact.  A row's screened argmin is the binary64 one unless a rival
 // lies within kThr of it.  In a wide segment the runner-up is kept.  Elsewhere
@@ -52,7 +55,9 @@
 
 namespace hjlo {
 
-constexpr int kDenseMaxWindow = 512;             // widest window (displacements)
+constexpr int kDenseMaxWindow = 3584;            // widest window (displacements; see kWide)
+constexpr int kScanWindow = 512;                 // widest window a lane scans alone for its pivot
+constexpr int kWide = 11;                        // the S of the banded search for wider ones
 constexpr int kFlat = 4;                         // the S of the flat search
 constexpr int kFlatMaxWindow = 96;               // widest window it takes (at most 128, its key numbers)
 constexpr unsigned kDensePad = 0x80000000u;      // table entries outside the window
@@ -65,14 +70,14 @@ enum { DENSE_BANDS = 0, DENSE_BRACKETS = 1, DENSE_BRUTE = 2 };
 // curvature it needs (2^kCurv key units).
 template <int S>
 struct DenseKey {
-    static constexpr int kBits = (S == kFlat) ? 7 : 5;
+    static constexpr int kBits = (S == kFlat) ? 7 : (S == kWide) ? 4 : 5;
     static constexpr unsigned kMask = (1u << kBits) - 1u, kThr = 2u * kMask + 6u, kFlag = kThr + kMask;
     static constexpr int kCurv = kBits + 3;
 };
 
 // Threads of a CTA at most, and CTAs an SM must hold (which caps registers).
-__host__ __device__ constexpr int dense_threads(int S) { return S <= 9 ? 256 : 512; }
-__host__ __device__ constexpr int dense_ctas(int S) { return S <= 9 ? 4 : 1; }
+__host__ __device__ constexpr int dense_threads(int S) { return S == kFlat ? 256 : 512; }
+__host__ __device__ constexpr int dense_ctas(int S) { return S == kFlat ? 4 : S <= 9 ? 2 : 1; }
 
 // Per-tile facts, in shared memory after the mbarrier.
 struct DenseInfo {
@@ -515,22 +520,74 @@ __device__ __forceinline__ void dense_tile(const CUtensorMap *tmap, const PassPa
                 if (p.vN && r == 0) flag(cl, 0);         // a row block's first row has no left neighbour
             }
         } else {
-        const int s0 = min(sub * S, NR), s1 = min(s0 + S, NR);
+        const int s0 = min(sub * S, NR), s1 = min(s0 + S, NR), nseg = (NR + S - 1) / S;
         const bool work = cl < tl.valid && s0 < s1;
-        const unsigned *lfx = fx + (work ? cl : 0) * p.lp;
-        OFF *lt = tt + (work ? cl : 0) * p.tp;
-        // ---- pivots: the first row of every segment over the whole window
+        const unsigned *lfx = fx + (cl < tl.valid ? cl : 0) * p.lp;
+        OFF *lt = tt + (cl < tl.valid ? cl : 0) * p.tp;
+        // ---- pivots: the first row of every segment over the whole window.  A
+        // row block is a periodic line of N points of which rows 0 .. NR - 1
+        // are wanted; rows NR and N - 1 are searched too, as the neighbours of
+        // the last one and the first.
+        auto last = [&] { return p.vN ? NR + lt[NR] : N + lt[0]; };       // source of the row after the last
         unsigned fl = 0;            // flagged rows, bit i: row s0 + i
         int jl = 0;
-        if (work) {
-            const unsigned *f = lfx + s0;
+        if constexpr (S == kWide) {
+            // wide windows (a warp's lanes hold one line's segments): the warp
+            // scans its first pivot's window together, then halves the
+            // distance between known pivots, the lanes between two of them
+            // sharing the sources between theirs
+            const int g0 = (sub >> 5) << 5;
+            const bool line = cl < tl.valid;
+            auto search = [&](int r, int j0, int j1, int i, int width, bool act, bool own) {
+                unsigned m = 0xffffffffu, m2 = 0xffffffffu;
+                int js = j0;
+                if (act) {
+                    const unsigned *f = lfx, *k = kd - r;
+                    const int jz = min(j1, r + weff - 1);
+#pragma unroll 4
+                    for (int j = max(j0, r) + i; j <= jz; j += width) {
+                        const unsigned c = f[j] + k[j];
+                        m2 = min(m2, max(m, c));
+                        js = (c < m) ? j : js;
+                        m = min(m, c);
+                    }
+                }
+                for (int o = 1; o < width; o <<= 1) {
+                    const unsigned om = __shfl_xor_sync(0xffffffffu, m, o), om2 = __shfl_xor_sync(0xffffffffu, m2, o);
+                    const int oj = __shfl_xor_sync(0xffffffffu, js, o);
+                    m2 = min(min(m2, om2), max(m, om));
+                    js = (om < m || (om == m && oj < js)) ? oj : js;
+                    m = min(m, om);
+                }
+                if (act && i == 0) {
+                    lt[r] = (OFF)(js - r);
+                    if (own && m2 - m <= Key::kThr) flag(cl, r);
+                }
+            };
+            search(g0 * S, 0, 0x3fffffff, lane, 32, line && g0 * S < NR, true);
+            if (p.vN) {                              // (see below)
+                if (g0 == 0) search(N - 1, 0, 0x3fffffff, lane, 32, line, false);
+                if (g0 == (nseg - 1) / 32 * 32) search(NR, 0, 0x3fffffff, lane, 32, line, false);
+            }
+            gsync();
+            for (int d = 16; d; d >>= 1) {
+                const int b = lane & ~(2 * d - 1), rl = (g0 + b) * S, r = rl + d * S, rr = rl + 2 * d * S;
+                const bool act = line && r < NR;
+                const int j0 = act ? rl + lt[rl] : 0, j1 = act ? (rr < NR ? rr + lt[rr] : last()) : 0;
+                search(r, j0, j1, lane - b, 2 * d, act, true);
+                __syncwarp();
+            }
+            if (work) jl = s0 + lt[s0];
+        } else if (work || (p.vN && cl < tl.valid && sub <= nseg + 1)) {
+            const int pr = work ? s0 : sub == nseg ? NR : N - 1;
+            const unsigned *f = lfx + pr;
             const uint4 *k4 = reinterpret_cast<const uint4 *>(kp);
             const int nch = (weff + 3) >> 2;
             unsigned m = 0xffffffffu, m2 = 0xffffffffu;
             int t = 0;
-            for (int c0 = 0; c0 < nch; c0 += 32) {
+            for (int c0 = 0; c0 < nch; c0 += (int)Key::kMask + 1) {
                 unsigned a[4] = {0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu};
-                const int c1 = min(c0 + 32, nch);
+                const int c1 = min(c0 + (int)Key::kMask + 1, nch);
 #pragma unroll 4
                 for (int c = c0; c < c1; ++c) {
                     const uint4 k = k4[c];
@@ -547,17 +604,15 @@ __device__ __forceinline__ void dense_tile(const CUtensorMap *tmap, const PassPa
                 t = (b < m) ? tb : t;
                 m = min(m, b);
             }
-            lt[s0] = (OFF)t;
-            jl = s0 + t;
-            if (m2 - m <= Key::kFlag) fl = 1u;
-            if (p.vN && sub == 0) fl = 1u;           // a row block's first row has no left neighbour
+            lt[pr] = (OFF)t;
+            if (work) jl = s0 + t;
+            if (work && m2 - m <= Key::kFlag) fl = 1u;
         }
         gsync();
         // ---- the rows between two pivots (lanes without a segment search a
         // line's first rows again and keep nothing)
         constexpr int kB = DenseBand<S>::kSources;
-        const int jr = (s1 < NR) ? s1 + lt[s1] : N + lt[0];
-        const bool next = !(p.vN && s1 == NR);       // row s1 is the next pivot (or row 0 one period on)
+        const int jr = (s1 < NR) ? s1 + lt[s1] : last();
         const int jc = min(jr, s1 + weff - 2);       // last source in any row's window
         const int span = work ? jc - jl + 1 : 1;
         {
@@ -605,9 +660,9 @@ __device__ __forceinline__ void dense_tile(const CUtensorMap *tmap, const PassPa
             const int from = act ? __ffs(rest) - 1 : lane;
             for (int i = 0; i < slots && wide; ++i) wide &= wide - 1;
             const int b0 = __shfl_sync(0xffffffffu, s0, from);
-            const int nrow = __shfl_sync(0xffffffffu, s1 - s0 + (next ? 1 : 0), from);     // rows to search
+            const int nrow = __shfl_sync(0xffffffffu, s1 - s0 + 1, from);  // rows to search
             const int j0 = __shfl_sync(0xffffffffu, jl, from);
-            const int j1 = __shfl_sync(0xffffffffu, next ? jr : jc, from);
+            const int j1 = __shfl_sync(0xffffffffu, jr, from);
             const int ln = __shfl_sync(0xffffffffu, cl, from);
             const int i0 = 2 * pair;                                 // rows b0 + i0, b0 + i0 + 1
             const int len = (j1 - j0 + H) / H;
@@ -617,10 +672,10 @@ __device__ __forceinline__ void dense_tile(const CUtensorMap *tmap, const PassPa
             if (act && i0 < nrow) {
                 const unsigned *f = fx + ln * p.lp;
                 const unsigned *kr = kd - (b0 + i0);                 // kr[j]: K for row b0 + i0
-                for (int jb = ja; jb < jz; jb += 32) {
+                for (int jb = ja; jb < jz; jb += (int)Key::kMask + 1) {
                     unsigned x[2] = {0xffffffffu, 0xffffffffu}, x2[2] = {0xffffffffu, 0xffffffffu};
                     unsigned k1 = kr[jb - 1];
-                    const int je = min(jb + 32, jz);
+                    const int je = min(jb + (int)Key::kMask + 1, jz);
 #pragma unroll 4
                     for (int j = jb; j < je; ++j) {
                         const unsigned fv = f[j] + (unsigned)(j - jb), k0 = kr[j];
@@ -657,7 +712,7 @@ __device__ __forceinline__ void dense_tile(const CUtensorMap *tmap, const PassPa
                     if (i >= nrow) continue;
                     const bool own = i > 0 && i < S && r < NR;       // a row of the segment, no pivot
                     if (own) wt[r] = (OFF)(js[b] - r);
-                    if (m2[b] - m[b] <= Key::kFlag) flag(ln, r < NR ? r : 0);
+                    if (m2[b] - m[b] <= Key::kFlag && (r < NR || !p.vN)) flag(ln, r < NR ? r : 0);
                 }
             }
         }
@@ -666,7 +721,7 @@ __device__ __forceinline__ void dense_tile(const CUtensorMap *tmap, const PassPa
             const int b = __ffs(fl) - 1;
             fl &= fl - 1;
             const int r = s0 + b;
-            flag(cl, r < s1 ? r : (s1 < NR) ? s1 : 0);
+            if (r < NR || !p.vN) flag(cl, r < s1 ? r : (s1 < NR) ? s1 : 0);
         }
         }
         gsync();
@@ -677,28 +732,70 @@ __device__ __forceinline__ void dense_tile(const CUtensorMap *tmap, const PassPa
             const int l0 = (grp << glog) >> p.log2lpl;               // the group's first line
             const int lines = min(max(gsize >> p.log2lpl, 1), tl.valid - l0);
             const int total = over ? max(lines, 0) * NR : (int)nf;
-            for (int x = gt; x < total; x += gsize) {
-                int l, r;
-                if (over) { l = x / NR; r = x - l * NR; l += l0; }
-                else { const unsigned e = queue[1 + x]; l = (int)(e >> 16); r = (int)(e & 0xffffu); }
-                OFF *ql = tt + l * p.tp;
-                const int lo = (r > 0) ? r - 1 + ql[r - 1] : (p.vN ? 0 : NR - 1 + ql[NR - 1] - N);
-                const int hi = (r + 1 < NR) ? r + 1 + ql[r + 1] : N + ql[0];
-                const DenseRow<T, LAYOUT> row{su, kr64, fx + l * p.lp + r, kd, N, p.hoff, p.log2C, l, r};
-                const int tlo = max(lo - r, 0), thi = min(hi - r, weff - 1);
-                const int t1 = ql[r];
-                const unsigned thr = row.key(t1) + Key::kThr;
-                unsigned mo = 0xffffffffu;                           // the best of the others
+            constexpr int kLong = 40;                                // more candidates: the warp's lanes share them
+            for (int x0 = gt & ~31; x0 < total; x0 += gsize) {
+                const int x = x0 + lane;
+                const bool has = x < total;
+                int l = 0, r = 0, tlo = 0, thi = -1, t1 = 0;
+                unsigned thr = 0;
+                DenseRow<T, LAYOUT> row{su, kr64, fx, kd, N, p.hoff, p.log2C, 0, 0};
+                if (has) {
+                    if (over) { l = x / NR; r = x - l * NR; l += l0; }
+                    else { const unsigned e = queue[1 + x]; l = (int)(e >> 16); r = (int)(e & 0xffffu); }
+                    const OFF *ql = tt + l * p.tp;
+                    // row -1 is row N - 1 one period back; the flat search has none of a
+                    // row block's outer rows
+                    const int lo = (r > 0) ? r - 1 + ql[r - 1] : (S == kFlat && p.vN) ? 0 : ql[N - 1] - 1;
+                    const int hi = (r + 1 < NR) ? r + 1 + ql[r + 1] : (S != kFlat && p.vN) ? NR + ql[NR] : N + ql[0];
+                    row.f = fx + l * p.lp + r;
+                    row.l = l;
+                    row.r = r;
+                    tlo = max(lo - r, 0);
+                    thi = min(hi - r, weff - 1);
+                    t1 = ql[r];
+                    thr = row.key(t1) + Key::kThr;
+                }
+                if (has && (S == kFlat || thi - tlo < kLong)) {
+                    unsigned mo = 0xffffffffu;                       // the best of the others
 #pragma unroll 4
-                for (int t = tlo; t < t1; ++t) mo = __viaddmin_u32(row.f[t], row.k[t], mo);
+                    for (int t = tlo; t < t1; ++t) mo = __viaddmin_u32(row.f[t], row.k[t], mo);
 #pragma unroll 4
-                for (int t = t1 + 1; t <= thi; ++t) mo = __viaddmin_u32(row.f[t], row.k[t], mo);
-                if (mo > thr) continue;
-                ++rescans;
-                Key2 best = key2_max();
-                int bt = t1;
-                row.exact(tlo, thi, 1, thr, best, bt);
-                ql[r] = (OFF)bt;
+                    for (int t = t1 + 1; t <= thi; ++t) mo = __viaddmin_u32(row.f[t], row.k[t], mo);
+                    if (mo <= thr) {
+                        ++rescans;
+                        Key2 best = key2_max();
+                        int bt = t1;
+                        row.exact(tlo, thi, 1, thr, best, bt);
+                        tt[l * p.tp + r] = (OFF)bt;
+                    }
+                }
+                if constexpr (S != kFlat) {
+                    unsigned lng = __ballot_sync(0xffffffffu, has && thi - tlo >= kLong);
+                    while (lng) {
+                        const int from = __ffs(lng) - 1;
+                        lng &= lng - 1;
+                        const int wl = __shfl_sync(0xffffffffu, l, from), wr = __shfl_sync(0xffffffffu, r, from);
+                        const int w0 = __shfl_sync(0xffffffffu, tlo, from), w1 = __shfl_sync(0xffffffffu, thi, from);
+                        const int wt = __shfl_sync(0xffffffffu, t1, from);
+                        const unsigned wthr = __shfl_sync(0xffffffffu, thr, from);
+                        const DenseRow<T, LAYOUT> wrow{su, kr64, fx + wl * p.lp + wr, kd, N, p.hoff, p.log2C, wl, wr};
+                        Key2 best = key2_max();
+                        int bt = wt, near = 0;
+#pragma unroll 4
+                        for (int t = w0 + lane; t <= w1; t += 32) near += (wrow.key(t) <= wthr) ? 1 : 0;
+                        if (__reduce_add_sync(0xffffffffu, near) <= 1) continue;
+                        wrow.exact(w0 + lane, w1, 32, wthr, best, bt);
+                        for (int o = 1; o < 32; o <<= 1) {
+                            const Key2 ob = key2_shfl_xor(best, o);
+                            const int ot = __shfl_xor_sync(0xffffffffu, bt, o);
+                            if (key2_less(ob, best) || (key2_eq(ob, best) && ot < bt)) { best = ob; bt = ot; }
+                        }
+                        if (lane == from) {
+                            ++rescans;
+                            tt[wl * p.tp + wr] = (OFF)bt;
+                        }
+                    }
+                }
             }
         }
         gsync();

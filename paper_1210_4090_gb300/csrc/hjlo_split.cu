@@ -188,6 +188,7 @@ __global__ void __launch_bounds__(kSplitThreads) split_classify(SplitParams p)
     const int b = (int)(blockIdx.x - line * p.B);
     const long long base = line_base(p, line);
     const int n = p.n, L = p.L;
+    pdl_wait();
     if (tid == 0) {
         s_fcv = INT_MAX;
         s_fcc = INT_MAX;
@@ -244,6 +245,7 @@ __global__ void __launch_bounds__(kSplitThreads) split_classify(SplitParams p)
         atomicMax(&s_mall, mx);
     }
     __syncthreads();
+    pdl_next();
     if (tid == 0) {
         const long long c = line * p.B + b;
         p.fcv[c] = (s_fcv == INT_MAX) ? -1 : s_fcv;
@@ -300,6 +302,8 @@ __global__ void __launch_bounds__(32 * kCutWarps) split_local_cut(SplitParams p)
     const int *fcv = p.fcv + line * p.B, *fcc = p.fcc + line * p.B;
     const int c0 = b * p.CH, c1 = c0 + p.CH, w0 = b * p.CW, L = p.L;
     unsigned *sv = s_v[wid], *sc = s_c[wid], *st = s_t[wid];
+    pdl_wait();
+    pdl_next();                                            // one CTA a line follows: it takes no room from these
 #pragma unroll
     for (int r = 0; r < (kMaxChunkWords + 32) / 32; ++r) {   // loads of all rounds issued together
         const int i = lane + 32 * r;
@@ -402,6 +406,8 @@ __global__ void __launch_bounds__(kStitchThreads) split_stitch(SplitParams p, in
     int *entry = p.entry + line * B, *lsm = p.lsm + line * B;
     int *cs = p.cs + line * B, *cm = p.cm + line * B;
     const int *F = p.F + line * p.Pl;
+    pdl_wait();
+    pdl_next();                                            // few CTAs: the next kernel's find room beside them
     if (stage) {
         // the walk's reads, all of them, from shared memory: local starts,
         // both rule bitmaps, the chunks' exits and first failing points
@@ -507,6 +513,7 @@ __global__ void __launch_bounds__(kSplitThreads) split_pieces(SplitParams p)
     const int *F = p.F + line * p.Pl;
     int *A = p.A + line * p.Pl;
     const int c0 = b * p.CH;
+    pdl_wait();
     if (tid == 0) s_count = (L == 1 && b == 0) ? 1ull : 0ull;   // a span of one point: one component
     __syncthreads();
     const int e = p.entry[cb];
@@ -555,6 +562,7 @@ __global__ void __launch_bounds__(kSplitThreads) split_pieces(SplitParams p)
         if (convex) atomicOr(&s_pk[(q - c0) >> 5], 1u << ((q - c0) & 31));
     }
     __syncthreads();
+    pdl_next();
     for (int i = tid; i < p.CW; i += nthr) p.pk[line * p.Wl + (long long)b * p.CW + i] = s_pk[i];
     if (tid == 0 && s_count) atomicAdd(&p.counters[CNT_COMPONENTS], s_count);
 }
@@ -670,6 +678,7 @@ __global__ void __launch_bounds__(kEmitThreads) split_emit(SplitParams p)
     const long long base = line_base(p, line);
     const unsigned *ts = p.ts + line * p.Wl, *pk = p.pk + line * p.Wl;
     const int *A = p.A + line * p.Pl;
+    pdl_wait();
 #pragma unroll 4
     for (int y = gy0 + tid; y <= gy1; y += nthr) {
         g[y - gy0] = p.src[base + lifted(p, y) * p.inner];
@@ -760,6 +769,7 @@ __global__ void __launch_bounds__(kEmitThreads) split_emit(SplitParams p)
         }
     }
     __syncthreads();
+    pdl_next();
     // values, potential term, stores
     for (int i = tid; i < nkeys; i += nthr) {
         const unsigned long long k = keys[i];
@@ -936,14 +946,16 @@ hjlo_status launch_split(const AxisPlan &ax, const void *src, void *dst, const d
     p.counters = counters;
     p.flags = flags;
     const long long chunks = p.lines * p.B;
-    split_classify<<<(unsigned)chunks, kSplitThreads, 0, st>>>(p);
-    split_local_cut<<<(unsigned)((chunks + kCutWarps - 1) / kCutWarps), 32 * kCutWarps, 0, st>>>(p);
     const size_t stage = sizeof(int) * 3 * (size_t)(p.Wl + p.B);
     const bool staged = stage <= kStitchStage;
-    split_stitch<<<(unsigned)p.lines, kStitchThreads, staged ? stage : 0, st>>>(p, staged ? 1 : 0);
-    split_pieces<<<(unsigned)chunks, kSplitThreads, 0, st>>>(p);
-    split_emit<<<(unsigned)(p.lines * p.nblk), kEmitThreads, ax.smem, st>>>(p);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_pdl(split_classify, (unsigned)chunks, kSplitThreads, 0, st, p);
+    if (e == cudaSuccess)
+        e = launch_pdl(split_local_cut, (unsigned)((chunks + kCutWarps - 1) / kCutWarps), 32 * kCutWarps, 0, st, p);
+    if (e == cudaSuccess)
+        e = launch_pdl(split_stitch, (unsigned)p.lines, kStitchThreads, staged ? stage : 0, st, p, staged ? 1 : 0);
+    if (e == cudaSuccess) e = launch_pdl(split_pieces, (unsigned)chunks, kSplitThreads, 0, st, p);
+    if (e == cudaSuccess)
+        e = launch_pdl(split_emit, (unsigned)(p.lines * p.nblk), kEmitThreads, ax.smem, st, p);
     if (e != cudaSuccess) return cuda_error(e, "decomposition kernel launch");
     return HJLO_OK;
 }

@@ -22,7 +22,8 @@
 //                maximum of F from its component's start (convex: Algorithm
 //                1's kernel pointer) or F itself (concave: alpha of Theorem
 //                th:ccc);
-//  5. emit       per block of outputs, every vertex of every component's
+//  5. emit       per block of outputs (several CTAs share the rows of one
+//                that many components reach), every vertex of every component's
 //                merged sequence that lands in the block -- each one a
 //                candidate fl(f(d) + g(y)) of the scheme -- is minimised into
 //                shared-memory keys, then stored with the potential term.
@@ -48,6 +49,9 @@ constexpr int kStitchThreads = 1024;
 constexpr int kCutWarps = 4;                 // chunks per CTA in the local cut (a warp each)
 constexpr int kMaxChunkWords = 128;          // chunks of at most 4096 points
 constexpr int kDefaultChunk = 1024;
+constexpr int kEmitParts = 24;               // CTAs that share a write-back block, at most
+constexpr int kEmitStarts = 16;              // component starts that one of them takes, at least
+constexpr long long kEmitShared = 1024;      // write-back blocks shared, when there are at most so many
 constexpr size_t kStitchStage = 200 * 1024;  // the stitch walk's data staged in shared memory up to this size
 
 struct SplitParams {
@@ -86,6 +90,8 @@ struct SplitParams {
     int *entry;                  // stitch: first true start that is a local start (-1: none)
     int *lsm;                    // stitch: last start taken by a single step (-1: none)
     int *cs, *cm;                // chain state at the chunk's first piece: start, max F so far
+    int *starts;                 // per write-back block: component starts among the points it reads; then their sum
+    int share;                   // the blocks' starts are counted and CTAs shared out by them
 };
 
 __device__ __forceinline__ long long line_base(const SplitParams &p, long long line)
@@ -189,6 +195,10 @@ __global__ void __launch_bounds__(kSplitThreads) split_classify(SplitParams p)
     const long long base = line_base(p, line);
     const int n = p.n, L = p.L;
     pdl_wait();
+    if (p.share)
+        for (long long i = (long long)blockIdx.x * blockDim.x + tid; i <= p.lines * p.nblk;
+             i += (long long)gridDim.x * blockDim.x)
+            p.starts[i] = 0;
     if (tid == 0) {
         s_fcv = INT_MAX;
         s_fcc = INT_MAX;
@@ -512,7 +522,7 @@ __global__ void __launch_bounds__(kSplitThreads) split_pieces(SplitParams p)
     const unsigned *ms = p.ms + line * p.Wl + (long long)b * p.CW;
     const int *F = p.F + line * p.Pl;
     int *A = p.A + line * p.Pl;
-    const int c0 = b * p.CH;
+    const int c0 = b * p.CH, n1 = p.n + 1;
     pdl_wait();
     if (tid == 0) s_count = (L == 1 && b == 0) ? 1ull : 0ull;   // a span of one point: one component
     __syncthreads();
@@ -565,6 +575,15 @@ __global__ void __launch_bounds__(kSplitThreads) split_pieces(SplitParams p)
     pdl_next();
     for (int i = tid; i < p.CW; i += nthr) p.pk[line * p.Wl + (long long)b * p.CW + i] = s_pk[i];
     if (tid == 0 && s_count) atomicAdd(&p.counters[CNT_COMPONENTS], s_count);
+    if (p.share && s_count) {
+        // the write-back blocks [x0, x0 + vR) that read this chunk's points (up to x0 + vR + n)
+        const int lo = max(0, c0 - n1) / p.vR;
+        const int hi = (int)min(p.nblk - 1, (long long)(c0 + p.CH - 1) / p.vR);
+        for (int k = lo + tid; k <= hi; k += nthr) {
+            atomicAdd(&p.starts[line * p.nblk + k], (int)s_count);
+            atomicAdd(&p.starts[p.lines * p.nblk], (int)s_count);
+        }
+    }
 }
 
 // ---------------------------------------------------------------- 5. emit
@@ -648,7 +667,24 @@ size_t emit_smem(int vR, int n)
            2 * sizeof(unsigned) * (span / 32 + 2);
 }
 
-// One CTA per block of vR outputs x in [x0, x1) of a line, z = x + n in
+// CTAs for a block with so many component starts among its points.  A start or
+// an end reaches up to a window of outputs, so where the cut alternates every
+// few points a few blocks hold nearly all vertices.  Such a block's rows are
+// divided among CTAs in proportion; what a CTA costs by itself (its points are
+// read and their spans counted, about as long as kEmitStarts components take)
+// and the mean over the blocks (below it nothing waits) say from where.  The
+// CTAs added, at most starts / mean - 1 a block, are never more than the
+// blocks.  Pendulum, 2^18 points, eta = dx: the first 200 steps 19.6 -> 12.7 ms,
+// the whole run 70.6 -> 65.5; of the smooth rest a pass costs what it did.
+__device__ __forceinline__ int emit_parts(const SplitParams &p, int starts, int sum)
+{
+    const int nb = (int)(p.lines * p.nblk);
+    const int each = max(kEmitStarts, (sum + nb - 1) / nb);
+    return max(1, min(min(kEmitParts, p.vR), (starts + each - 1) / each));
+}
+
+// One CTA per block of vR outputs x in [x0, x1) of a line, or several that
+// share its rows (emit_parts; the second half of the grid), z = x + n in
 // [zlo, zhi).  Vertices reaching the block come from points y in
 // [x0, x1 + n) and pieces p in [x0 - 1, x1 + n), all staged in shared
 // memory; the point vertices are spread evenly over the threads by a scan
@@ -658,10 +694,47 @@ __global__ void __launch_bounds__(kEmitThreads) split_emit(SplitParams p)
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_wsum[32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nthr = blockDim.x, nw = nthr >> 5;
-    const long long line = blockIdx.x / p.nblk;
-    const long long blk = blockIdx.x - line * p.nblk;
+    const long long nb = p.lines * p.nblk;
+    long long cta = blockIdx.x;
+    int part = 0, parts = 1;
+    pdl_wait();
+    if (p.share) {
+        const int sum = p.starts[nb];
+        if (cta < nb) {
+            parts = emit_parts(p, p.starts[cta], sum);
+        } else {
+            // the (cta - nb)-th added CTA: blocks in order, one a thread
+            __shared__ int s_cta, s_part, s_parts;
+            const int mine = (tid < nb) ? emit_parts(p, p.starts[tid], sum) : 1;
+            int incl = mine - 1;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += u;
+            }
+            if (lane == 31) s_wsum[warp] = incl;
+            if (tid == 0) s_cta = -1;
+            __syncthreads();
+            for (int w = 0; w < warp; ++w) incl += s_wsum[w];
+            const int want = (int)(cta - nb);
+            if (want < incl && want >= incl - (mine - 1)) {
+                s_cta = tid;
+                s_part = want - (incl - (mine - 1)) + 1;
+                s_parts = mine;
+            }
+            __syncthreads();
+            if (s_cta < 0) return;
+            cta = s_cta;
+            part = s_part;
+            parts = s_parts;
+        }
+    }
+    const long long line = cta / p.nblk;
+    const long long blk = cta - line * p.nblk;
     const int n = p.n, L = p.L;
-    const int x0 = (int)(blk * p.vR), x1 = (int)min((long long)x0 + p.vR, p.N);
+    const int rows = (p.vR + parts - 1) / parts;
+    const int x0 = (int)(blk * p.vR) + part * rows;
+    const int x1 = (int)min((long long)min(x0 + rows, (int)(blk * p.vR) + p.vR), p.N);
+    if (x0 >= x1) return;                                              // the whole CTA
     const int zlo = x0 + n, zhi = x1 + n, nkeys = x1 - x0;
     const int gy0 = max(0, x0 - 1), gy1 = min(L - 1, x1 + n);        // staged points [gy0, gy1]
     const int ylo = x0, yhi = min(L - 1, x1 + n - 1);                  // points [ylo, yhi]
@@ -678,7 +751,6 @@ __global__ void __launch_bounds__(kEmitThreads) split_emit(SplitParams p)
     const long long base = line_base(p, line);
     const unsigned *ts = p.ts + line * p.Wl, *pk = p.pk + line * p.Wl;
     const int *A = p.A + line * p.Pl;
-    pdl_wait();
 #pragma unroll 4
     for (int y = gy0 + tid; y <= gy1; y += nthr) {
         g[y - gy0] = p.src[base + lifted(p, y) * p.inner];
@@ -851,7 +923,7 @@ namespace {
 
 // Scratch layout of an axis (offsets into d_split; every array 16-byte aligned).
 struct SplitLayout {
-    size_t cv, cc, ts, ms, pk, rk, F, A, wmax, chunk[10], bytes;
+    size_t cv, cc, ts, ms, pk, rk, F, A, wmax, chunk[10], starts, bytes;
 };
 SplitLayout split_layout(const AxisPlan &ax)
 {
@@ -874,6 +946,7 @@ SplitLayout split_layout(const AxisPlan &ax)
     s.A = take(4 * pieces);
     s.wmax = take(4 * words);
     for (int i = 0; i < 10; ++i) s.chunk[i] = take(4 * chunks);
+    s.starts = take(4 * (lines * (size_t)ax.dnblk + 1));
     s.bytes = off;
     return s;
 }
@@ -914,6 +987,8 @@ SplitParams split_params(const AxisPlan &ax)
     p.F = reinterpret_cast<int *>(w + lay.F);
     p.A = reinterpret_cast<int *>(w + lay.A);
     p.wmax = reinterpret_cast<int *>(w + lay.wmax);
+    p.starts = reinterpret_cast<int *>(w + lay.starts);
+    p.share = p.lines * p.nblk <= kEmitShared;
     int **chunk_arrays[10] = {&p.fcv, &p.fcc, &p.mall, &p.X, &p.lastl, &p.mtl, &p.entry, &p.lsm, &p.cs, &p.cm};
     for (int i = 0; i < 10; ++i) *chunk_arrays[i] = reinterpret_cast<int *>(w + lay.chunk[i]);
     return p;
@@ -955,7 +1030,7 @@ hjlo_status launch_split(const AxisPlan &ax, const void *src, void *dst, const d
         e = launch_pdl(split_stitch, (unsigned)p.lines, kStitchThreads, staged ? stage : 0, st, p, staged ? 1 : 0);
     if (e == cudaSuccess) e = launch_pdl(split_pieces, (unsigned)chunks, kSplitThreads, 0, st, p);
     if (e == cudaSuccess)
-        e = launch_pdl(split_emit, (unsigned)(p.lines * p.nblk), kEmitThreads, ax.smem, st, p);
+        e = launch_pdl(split_emit, (unsigned)(p.lines * p.nblk * (p.share ? 2 : 1)), kEmitThreads, ax.smem, st, p);
     if (e != cudaSuccess) return cuda_error(e, "decomposition kernel launch");
     return HJLO_OK;
 }

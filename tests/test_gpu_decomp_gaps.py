@@ -1,8 +1,9 @@
 """The whole-period decomposition's emission where points with many vertices
 and long stretches without any (the inside of concave components) alternate in
 a write-back block: rough stretches at the line's ends, across its seam and
-between blocks, one rough line among smooth ones, blocks of few rows.  Bit for
-bit the oracle's method, with its number of components."""
+between blocks, one rough line among smooth ones.  Several CTAs share the rows
+of a block that many components reach; blocks of few rows, of rows that do not
+divide, and more blocks than are shared (rows 1).  Bit for bit the oracle's method, with its number of components."""
 import numpy as np
 import pytest
 

@@ -455,7 +455,7 @@ __global__ void __launch_bounds__(kStitchThreads) split_stitch(SplitParams p, in
                 s = X[b];
             } else {
                 if (lane == 0) {
-                    ms[s >> 5] |= 1u << (s & 31);
+                    atomicOr(&ms[s >> 5], 1u << (s & 31));    // its result unused: the walk does not wait for it
                     lsm[b] = s;
                 }
                 s = warp_next_start(p, cv, cc, fcv, fcc, s);
@@ -469,12 +469,17 @@ __global__ void __launch_bounds__(kStitchThreads) split_stitch(SplitParams p, in
     // joined its local cut ends with it; one that did not, with its last
     // single step (its max of F taken here, a warp per chunk, into the local
     // cut's slots, which that chunk no longer needs)
-    for (int b = warp; b < B; b += nw) {
-        if (entry[b] >= 0 || lsm[b] < 0) continue;
-        const int mt = warp_tail_max(p, F, p.wmax + line * p.Wl, lsm[b], (b + 1) * p.CH);
-        if (lane == 0) {
-            lastl[b] = lsm[b];
-            mtl[b] = mt;
+    for (int b0 = 0; b0 < B; b0 += 32 * nw) {
+        const int c = b0 + warp + nw * lane;               // the warp's chunks, looked at together
+        const int at = (c < B && entry[c] < 0) ? lsm[c] : -1;
+        for (unsigned todo = __ballot_sync(0xffffffffu, at >= 0); todo; todo &= todo - 1u) {
+            const int l = __ffs(todo) - 1, b = b0 + warp + nw * l;
+            const int from = __shfl_sync(0xffffffffu, at, l);
+            const int mt = warp_tail_max(p, F, p.wmax + line * p.Wl, from, (b + 1) * p.CH);
+            if (lane == 0) {
+                lastl[b] = from;
+                mtl[b] = mt;
+            }
         }
     }
     __syncthreads();

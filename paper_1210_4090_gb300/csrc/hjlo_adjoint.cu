@@ -23,6 +23,12 @@
 // term's derivative Vbar -= h * ubar^{n+1} is taken by the step's first
 // reverse pass as it loads ubar.
 //
+// What bounds it: the latency of a pass's four phases (load, check, inversion,
+// gather), so each is kept short: a thread stays on its line, which takes the
+// divisions by the line length out of every loop, and dk/dP comes from a table
+// in shared memory instead of a conversion and a product on the binary64 pipe
+// per target (512^2, 128 steps, a whole gradient: 7750 -> 7273 us).
+//
 // Memory: forward states are checkpointed every S steps; each segment is
 // recomputed once with argmin recording (S x ndim x npts int32) and then
 // reversed.

@@ -46,9 +46,9 @@
 // first (1-4 % of the rows on the solver's fields).
 //
 // What bounds it.  The pipe of the 32-bit minimum, logic and shift instructions
-// (64 lanes a clock and SM, about 60 % busy), shared-memory words and issue
-// slots (70 %) are within a factor of 1.3 of one another; staging and write-back
-// alone take 68 of the 157 us on the 256^3 grid.
+// (64 lanes a clock and SM, 62-68 % busy), shared-memory words (62 %) and issue
+// slots (65 %) are within a factor of 1.1 of one another; staging and write-back
+// alone take 68 of the 155 us on the 256^3 grid.
 #pragma once
 
 #include "hjlo_device.cuh"

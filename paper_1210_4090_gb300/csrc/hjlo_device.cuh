@@ -17,7 +17,8 @@
 // is ascending lifted source, so a strict '<' scan keeps the smallest source
 // among equal values (the library's tie rule).
 //
-// MONGE search.  u[j] + k[i-j] is a Monge matrix with margin
+// MONGE search (by divide and conquer: for the tiles that the register-tile
+// searches of hjlo_dense.cuh leave, see dense_segment).  u[j] + k[i-j] is a Monge matrix with margin
 // a = min second difference of k > 0 (k convex, hypothesis (i)): the leftmost
 // row argmin is non-decreasing in i, and along the periodic line
 // argmin(i+N) = argmin(i) + N.  Lane g of the line's lpl lanes owns the rows

@@ -879,8 +879,8 @@ hjlo_status split_allow_smem()
 // [64, 4096], for tests that want many chunks on short lines or few on long
 // ones); write-back blocks of about one per SM over all lines, at least 256
 // rows (HJLO_DECOMP_SPLIT_ROWS sets them), fewer while their shared memory
-// does not fit (the 2^18-point pendulum at eta = dx, a whole run: 152
-// blocks of 1725 rows 53 us per pass, 304 of 862 55 us, 76 of 3450 73 us).
+// does not fit (the 2^18-point pendulum at eta = dx, a whole run, one CTA a
+// block: 152 blocks of 1725 rows 53 us per pass, 304 of 862 55, 76 of 3450 73).
 hjlo_status shape_split(AxisPlan &ax, size_t smem_optin, int num_sms)
 {
     smem_optin = (smem_optin > kStaticReserve) ? smem_optin - kStaticReserve : 0;

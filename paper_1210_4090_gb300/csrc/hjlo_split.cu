@@ -48,11 +48,11 @@ constexpr int kEmitThreads = 1024;
 constexpr int kStitchThreads = 1024;
 constexpr int kCutWarps = 4;                 // chunks per CTA in the local cut (a warp each)
 constexpr int kMaxChunkWords = 128;          // chunks of at most 4096 points
-constexpr int kDefaultChunk = 1024;
+constexpr int kDefaultChunk = 512;
 constexpr int kEmitParts = 24;               // CTAs that share a write-back block, at most
 constexpr int kEmitStarts = 16;              // component starts that one of them takes, at least
 constexpr long long kEmitShared = 1024;      // write-back blocks shared, when there are at most so many
-constexpr size_t kStitchStage = 200 * 1024;  // the stitch walk's data staged in shared memory up to this size
+constexpr size_t kStitchStage = 212 * 1024;  // the stitch walk's data staged in shared memory up to this size
 
 struct SplitParams {
     const double *src;
@@ -875,12 +875,16 @@ hjlo_status split_allow_smem()
     return e == cudaSuccess ? HJLO_OK : cuda_error(e, "cudaFuncSetAttribute(split)");
 }
 
-// Chunks of kDefaultChunk points (HJLO_DECOMP_CHUNK: a multiple of 32 in
-// [64, 4096], for tests that want many chunks on short lines or few on long
-// ones); write-back blocks of about one per SM over all lines, at least 256
-// rows (HJLO_DECOMP_SPLIT_ROWS sets them), fewer while their shared memory
-// does not fit (the 2^18-point pendulum at eta = dx, a whole run, one CTA a
-// block: 152 blocks of 1725 rows 53 us per pass, 304 of 862 55, 76 of 3450 73).
+// Chunks of kDefaultChunk points: shorter ones shorten the serial cut of a
+// chunk, more of them lengthen the stitch (400 steps at eta = dx, chunks of
+// 384 / 512 / 640 / 1024 points: 8192 points 8.6 / 8.7 / 9.2 / 9.5 ms, 65536
+// 11.4 / 11.2 / 11.9 / 12.4, 2^18 21.8 / 20.0 / 20.3 / 20.1; 1635 steps on 2^18
+// with 256 / 512 / 1024 / 2048: 70 / 60 / 62.5 / 73).  HJLO_DECOMP_CHUNK sets
+// them (a multiple of 32 in [64, 4096]), for tests that want many chunks on
+// short lines or few on long ones.  Write-back blocks of about one per SM over
+// all lines, at least 256 rows (HJLO_DECOMP_SPLIT_ROWS sets them), fewer while
+// their shared memory does not fit (the 2^18-point pendulum at eta = dx, a
+// whole run: 152 blocks of 1725 rows 60 ms, 202 of 1300 67, 304 of 862 70).
 hjlo_status shape_split(AxisPlan &ax, size_t smem_optin, int num_sms)
 {
     smem_optin = (smem_optin > kStaticReserve) ? smem_optin - kStaticReserve : 0;

@@ -62,7 +62,7 @@ constexpr int kFlat = 4;                         // the S of the flat search
 constexpr int kFlatMaxWindow = 96;               // widest window it takes (at most 128, its key numbers)
 constexpr unsigned kDensePad = 0x80000000u;      // table entries outside the window
 constexpr int kDenseLow = 16, kDenseHigh = 32;   // padding of the table K
-constexpr int kDenseOver = 16;                   // halo entries read past its end (full bands)
+constexpr int kDenseOver = 16;                   // halo entries past N + weff - 1 (row N's last, full bands)
 enum { DENSE_BANDS = 0, DENSE_BRACKETS = 1, DENSE_BRUTE = 2 };
 
 // Low key bits (a source's number in its band; the displacement's in the flat
@@ -413,13 +413,14 @@ __device__ __forceinline__ void dense_tile(const CUtensorMap *tmap, const PassPa
             if (!isfinite(umax - umin) || !isfinite(cmax) || q > 900 || !(p.curv > __dmul_ru(cmax, 0x1p-49)))
                 mode = DENSE_BRUTE;
         }
-        // ---- keys: the halo (its last weff - 1 entries repeat the first ones
-        // one period later; a few more are read by full bands and never win)
-        // and the table
+        // ---- keys: the halo (its first weff entries repeat one period later:
+        // row N, row 0's image, is searched with the last segment when that is
+        // a wide one, over its whole window; a few more entries are read by full
+        // bands, beside no displacement of the window) and the table
         if (mode != DENSE_BRUTE) {
             const double magic = key_magic(q);
             const unsigned fref = info->fref, kref = info->kref;
-            const int dup = weff - 1;
+            const int dup = weff;
             if (mine) {
                 const T *x = (LAYOUT == LAYOUT_CONTIG) ? su + l * N + first : su + tid;
                 const int xs = (LAYOUT == LAYOUT_CONTIG) ? lpl : nthr;
@@ -441,7 +442,7 @@ __device__ __forceinline__ void dense_tile(const CUtensorMap *tmap, const PassPa
                     for (int b = 0; b < 4; ++b) put(v[b], pos + b * step, b & 1);
                 }
                 for (; pos < N; pos += step, x += xs) put(*x, pos, false);
-                for (int i = first; i < kDenseOver; i += step) lfn[dup + i] = 0u;
+                for (int i = first; i < kDenseOver - 1; i += step) lfn[dup + i] = 0u;
             }
             for (int i = tid; i < kDenseLow + weff + kDenseHigh; i += nthr) {
                 const int t = i - kDenseLow;

@@ -39,8 +39,16 @@
 // each row keeps four minima, one per source number mod 4: a rival of another
 // class shows in them, and one of the same class is 4 or more sources away;
 // since it gains at least 2^kCurv - kFlag on the nearer sources with each row,
-// the neighbouring row's source has passed it, so it shows as a step of 4 or
-// more between two rows' sources.  Rows flagged by either are searched again
+// the neighbouring row's source (the row before's for a rival to the left, the
+// row after's for one to the right) has passed it, so it shows as a step of 4 or
+// more between two rows' sources.  Every pair of neighbours is looked at: two
+// rows of a lane, a lane's last row and the next lane's first, and round the
+// end of the line: row N - 1 and row 0's image one period on (when the last
+// segment is a wide one, the image row is searched with it, over the whole of
+// its window), or for row blocks row NR - 1 and row NR, and row -1 (row N - 1
+// of the block's periodic line) and row 0.  The flat search, which has none of
+// a row block's outer rows, flags row 0 of every block instead; wide windows'
+// pivots keep their runner-up.  Rows flagged by either are searched again
 // between their neighbours' sources (a rival further out would have taken the
 // neighbour), survivors of the screen compared in binary64, smallest source
 // first (1-4 % of the rows on the solver's fields).
@@ -610,6 +618,9 @@ __device__ __forceinline__ void dense_tile(const CUtensorMap *tmap, const PassPa
             if (work && m2 - m <= Key::kFlag) fl = 1u;
         }
         gsync();
+        // a row block's first row and the one before it: on whole lines the last
+        // segment sees this step
+        if (S != kWide && p.vN && work && sub == 0 && lt[0] - (lt[N - 1] - 1) >= 4) fl |= 1u;
         // ---- the rows between two pivots (lanes without a segment search a
         // line's first rows again and keep nothing)
         constexpr int kB = DenseBand<S>::kSources;

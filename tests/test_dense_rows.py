@@ -153,6 +153,8 @@ class Line:
                 flags[g] |= fl
             if block:
                 lt[N - 1], lt[NR] = self.scan_pivot(N - 1)[0], self.scan_pivot(NR)[0]
+                if lt[0] - (lt[N - 1] - 1) >= 4:
+                    flags[0] |= 1
         for g in range(nseg):
             s0, s1 = g * S, min(g * S + S, NR)
             jl, jr = s0 + lt[s0], s1 + lt[s1] if s1 < NR else last()
@@ -224,7 +226,7 @@ def _check(u, k, NR, S):
 
 
 @pytest.mark.parametrize("ends", [True, False], ids=["ends", "anywhere"])
-@pytest.mark.parametrize("block", [False], ids=["line"])
+@pytest.mark.parametrize("block", [False, True], ids=["line", "block"])
 @pytest.mark.parametrize("S", [FLAT, 9, 13, WIDE])
 def test_close_rivals_are_compared(S, block, ends):
     rng = np.random.default_rng([S, block, ends])

@@ -53,3 +53,21 @@ def test_whole_lines(N, W, lanes, ends, monkeypatch):
     val, ram = _expect(u, k, W)
     assert np.array_equal(got.view(np.int64), val.view(np.int64))
     assert np.array_equal(am, ram)
+
+
+@pytest.mark.parametrize("N,W,rows", [(4100, 40, 300), (4100, 100, 400), (4100, 100, 700), (9100, 400, 900)],
+                         ids=["flat", "9", "13", "11"])
+def test_first_rows_of_row_blocks(N, W, rows, monkeypatch):
+    rng = np.random.default_rng([N, W, rows])
+    h, w, k = 0.02, 2 * W + 1, _table(2 * W + 1, 1.0 / N, 0.02)
+    u = np.empty((70, N))
+    for i in range(len(u)):
+        parts = [_rivals(rng, rows + w - 1, k, rows, True)[:w + 8] for _ in range(N // rows)]
+        u[i] = max(q.max() for q in parts)
+        for b, q in enumerate(parts):
+            u[i, (b * rows - W + np.arange(w + 8)) % N] = q
+    got, am, info = _run(u, W, h, monkeypatch, {"HJLO_BLOCK_ROWS": rows})
+    assert info["row_blocks"][1] > 1 and info["block_rows"][1] == rows
+    val, ram = _expect(u, k, W)
+    assert np.array_equal(got.view(np.int64), val.view(np.int64))
+    assert np.array_equal(am, ram)

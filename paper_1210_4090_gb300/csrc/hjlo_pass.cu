@@ -341,28 +341,38 @@ static hjlo_status shape_lines(AxisPlan &ax, int esize, int algo, int num_sms, s
 // lines than half the SMs; they hold about one SM's share of the rows, at
 // least weff - 1 (a block stages vR + weff - 1 points for vR rows; twice that
 // left half as many SMs at work: 8192-point line, 291 displacements, 289 steps
-// 2.59 against 2.38 ms) and at most what fits.  Brute force, whose rows cost weff candidates each
+// 2.59 against 2.38 ms) and at most what fits.  `tiles`: for the register-tile
+// searches, whose shared memory is a little more; blocks that do not get them
+// are sized for divide and conquer (shape_launch), which takes 2 (weff - 1)
+// rows of windows above kTwoWindows (one line of 20000 points, 2401
+// displacements: 2400 rows 102 us a pass, 4800 68; 2^18 points, 3801: 3800 rows
+// 267, 7600 184; 8192 points, 1601: 1600 rows 33, 3200 38).
+// Brute force, whose rows cost weff candidates each
 // against one staged point, also takes blocks for wider windows (up to the
 // full torus window) on an axis with few lines, from one row per block: a
 // lone line then spreads over many SMs instead of one SM's binary64 pipe.
 // A hint (hinted > 0) replaces the share, within [weff - 1 (brute: 1), what
 // fits].
+constexpr int kTwoWindows = 2048;
 static long long block_rows(const AxisPlan &ax, int esize, int algo, int num_sms, size_t smem_optin,
-                            long long hinted)
+                            long long hinted, bool tiles)
 {
     const long long N = ax.N, w = ax.weff, lines = ax.outer;
     const bool brute = (algo == KALGO_BRUTE);
     if (ax.inner != 1 || (4 * w > N && !brute)) return 0;
-    // shared memory per staged point and per window entry (layout_smem)
-    const long long per_pt = esize + 2 + ((algo == KALGO_MONGE) ? 5 : 0);
-    const long long per_w = 8 + ((algo == KALGO_MONGE) ? 12 : 0);
-    const long long room = (long long)smem_optin - 1024 - per_w * w;
-    const long long fit_pts = room > 0 ? room / per_pt : 0;         // staged points that fit
-    const bool fits = N + w <= fit_pts;
+    // staged points that fit, from the bytes per point and per window entry (layout_smem)
+    const auto fit = [&](long long per_pt, long long per_w) {
+        const long long room = (long long)smem_optin - 1024 - per_w * w;
+        return room > 0 ? room / per_pt : 0;
+    };
+    const long long least = brute ? 1 : std::max(1LL, w - 1);
+    const long long whole = brute ? fit(esize + 2, 8) : fit(esize + 6, 16);
+    const long long fit_pts = tiles ? fit(esize + 2 + (w > kScanWindow ? 6 : 5), 20) : whole;
+    const bool fits = N + w <= whole;
     if (fits && 2 * lines >= num_sms) return 0;
     if (brute && 4 * w > N && !(2 * lines < num_sms)) return 0;     // wide windows: few lines only
-    const long long least = brute ? 1 : std::max(1LL, w - 1);
-    long long vR = std::max(brute ? 1 : w - 1, (N * lines + num_sms - 1) / num_sms);
+    long long vR = brute ? 1 : (!tiles && w > kTwoWindows) ? 2 * (w - 1) : w - 1;
+    vR = std::max(vR, (N * lines + num_sms - 1) / num_sms);
     if (hinted > 0) vR = std::max(hinted, least);
     vR = std::min(vR, fit_pts - (w - 1));
     vR = std::min(vR, N - (w - 1));                                 // a block never spans the line
@@ -379,8 +389,9 @@ hjlo_status shape_launch(AxisPlan &ax, int esize, int algo, int num_sms, size_t 
     ax.rows = 0;
     if ((algo == KALGO_MONGE || algo == KALGO_BRUTE) && row_blocks) {
         const ShapeHints hint = hints ? *hints : env_hints();
-        const long long vR = block_rows(ax, esize, algo, num_sms, smem_optin, hint.block_rows);
-        if (vR > 0) {
+        for (int tiles = (algo == KALGO_MONGE && ax.weff <= kDenseMaxWindow) ? 1 : 0; tiles >= 0; --tiles) {
+            const long long vR = block_rows(ax, esize, algo, num_sms, smem_optin, hint.block_rows, tiles != 0);
+            if (vR <= 0) continue;
             AxisPlan v = ax;
             v.N = vR + ax.weff - 1;
             v.vblocks = (ax.N + vR - 1) / vR;
@@ -388,6 +399,7 @@ hjlo_status shape_launch(AxisPlan &ax, int esize, int algo, int num_sms, size_t 
             v.hoff = 0;
             v.rows = vR;                      // only the block's own rows are searched
             hjlo_status s = shape_lines(v, esize, algo, num_sms, smem_optin, 1, hints);
+            if (tiles && (s != HJLO_OK || !v.dense)) continue;       // blocks for divide and conquer
             if (s != HJLO_OK) return s;
             // launch fields from the block lines; geometry and tables stay the axis's
             AxisPlan r = v;

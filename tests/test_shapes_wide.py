@@ -1,0 +1,55 @@
+"""Launch shapes of the monotone search's row blocks on the host: windows that a
+block of at least weff - 1 rows holds by divide and conquer are taken, whatever
+the register-tile searches would need; blocks sized for those are searched by
+them; long lines that fit one CTA are launched whole when there are enough."""
+import pytest
+
+from paper_1210_4090_gb300 import hjlo
+
+SMEM = 232448
+
+
+@pytest.fixture(autouse=True)
+def _no_overrides(monkeypatch):
+    for k in ("HJLO_LANES_PER_LINE", "HJLO_LINES_PER_TILE", "HJLO_OFFLOAD", "HJLO_BLOCK_ROWS"):
+        monkeypatch.delenv(k, raising=False)
+
+
+def _holds(weff, esize):
+    """Whether divide and conquer holds weff - 1 rows: their span of 2 (weff - 1) points at esize + 6 bytes
+    each (value, screened value, argmin offset) and 16 a displacement, less 1 KB of padding."""
+    return 2 * (weff - 1) <= (SMEM - 1024 - 16 * weff) // (esize + 6)
+
+
+@pytest.mark.parametrize("esize", [8, 4])
+@pytest.mark.parametrize("lines", [1, 40, 1024])
+def test_wide_windows_are_taken(lines, esize):
+    taken = []
+    for weff in range(3001, 6602, 100):
+        N = 4 * weff + 7
+        if not _holds(weff, esize):
+            with pytest.raises(hjlo.HjloError):
+                hjlo.shape_query(1 << 18, 1, weff, esize)
+            continue
+        s = hjlo.shape_query(max(N, 1 << 16), lines, weff, esize)
+        assert s["row_blocks"] > 1 and s["block_rows"] >= weff - 1, (weff, s)
+        taken.append(weff)
+    assert max(taken) >= (5200 if esize == 8 else 6300)
+
+
+@pytest.mark.parametrize("N,lines,weff", [(10000, 1024, 2401), (12000, 300, 1601), (14000, 200, 881)])
+def test_long_lines_that_fit_are_whole(N, lines, weff):
+    assert hjlo.shape_query(N, lines, weff)["row_blocks"] == 1
+
+
+@pytest.mark.parametrize("N,weff,rows,seg", [
+    (1 << 18, 3271, 3270, 11), (65536, 1601, 1600, 11),    # weff - 1 rows, searched in segments of 11
+    (1 << 18, 201, 1725, 9), (65536, 291, 432, None),      # one SM's share; few lanes: divide and conquer
+    (20000, 2401, 4800, None), (1 << 18, 3801, 7600, None),      # divide and conquer: 2 (weff - 1) rows
+    (8192, 291, 290, None)])
+def test_block_rows(N, weff, rows, seg):
+    s = hjlo.shape_query(N, 1, weff)
+    assert s["block_rows"] == rows, s
+    if seg:
+        assert s["segment_rows"] == seg, s
+    assert s["threads"] >= (128 if weff > 512 else 32), s

@@ -71,7 +71,6 @@ constexpr int kFlatMaxWindow = 96;               // widest window it takes (at m
 constexpr unsigned kDensePad = 0x80000000u;      // table entries outside the window
 constexpr int kDenseLow = 16, kDenseHigh = 32;   // padding of the table K
 constexpr int kDenseOver = 16;                   // halo entries past N + weff - 1 (row N's last, full bands)
-enum { DENSE_BANDS = 0, DENSE_BRACKETS = 1, DENSE_BRUTE = 2 };
 
 // Low key bits (a source's number in its band; the displacement's in the flat
 // search), the screen's error between two sums without and with them, and the
@@ -92,7 +91,7 @@ struct DenseInfo {
     int kmin, kmax;             // extremes of the tile (float_key)
     unsigned fref, kref;        // keys' references: below min u and -max|k| at 2^q
     int q;                      // key unit 2^q (32 of them: 2^(q+5))
-    int mode;                   // DENSE_*
+    int ok;                     // the screen holds: finite values, enough curvature
 };
 
 // Sources of a bracket that one lane searches.
@@ -151,17 +150,6 @@ __device__ __forceinline__ int key_hi<float>(int key)
 {
     return __double2hiint(widen(__int_as_float(key ^ ((key >> 31) & 0x7fffffff))));
 }
-// A binary64 bound on the values from the extreme's key.
-template <typename T>
-__device__ __forceinline__ double key_bound(int key, bool lower);
-template <>
-__device__ __forceinline__ double key_bound<double>(int key, bool lower) { return hikey_bound(key, lower); }
-template <>
-__device__ __forceinline__ double key_bound<float>(int key, bool)
-{
-    return (double)__int_as_float(key ^ ((key >> 31) & 0x7fffffff));
-}
-
 // +-significand(h) 2^(e(h) - 1043 - q), h the high word of a binary64 number of
 // either sign, rounded down (the low word as large as it can be for a negative
 // one), modulo 2^32: a reference below every key of values from that number on.
@@ -177,8 +165,8 @@ __device__ __forceinline__ unsigned key_below(int h, int q)
     return (m ^ neg) - neg;
 }
 
-// Scale and mode of a tile from its extremes' high words (a lower and an upper
-// bound) with 32-bit instructions only, by one thread: the binary64 pipe is
+// Scale of a tile, and whether the screen holds there, from its extremes' high
+// words (a lower and an upper bound) with 32-bit instructions only, by one thread: the binary64 pipe is
 // busy with other CTAs' sums, and a chain of a dozen dependent operations on it
 // took 2200 clocks of a tile's 25000.
 __device__ __forceinline__ void dense_scale(int hmin, int hmax, double kmax, double curv, int cbits, DenseInfo *info)
@@ -197,7 +185,7 @@ __device__ __forceinline__ void dense_scale(int hmin, int hmax, double kmax, dou
     // than binary64 ties need
     const bool ok = E < 0x7ff && q <= 900 && hc > 0 && (hc >> 20) - 1023 >= q + cbits;
     info->q = q;
-    info->mode = ok ? DENSE_BANDS : DENSE_BRACKETS;
+    info->ok = ok ? 1 : 0;
     info->fref = key_below(hmin, q);
     info->kref = key_below(hk | (int)0x80000000, q);
 }
@@ -275,77 +263,19 @@ struct DenseRow {
                 if (key2_less(c, best)) { best = c; bt = t; }
             }
     }
-    // one lane alone: screened minimum and runner-up, then binary64 if needed
-    __device__ __forceinline__ int search(int tlo, int thi, unsigned tol, int &rescans) const
-    {
-        unsigned m = 0xffffffffu, m2 = 0xffffffffu;
-        int bt = tlo;
-        for (int t = tlo; t <= thi; ++t) {
-            const unsigned c = key(t);
-            m2 = min(m2, max(m, c));
-            bt = (c < m) ? t : bt;
-            m = min(m, c);
-        }
-        if (m2 - m > tol) return bt;
-        ++rescans;
-        Key2 best = key2_max();
-        exact(tlo, thi, 1, m + tol, best, bt);
-        return bt;
-    }
 };
 
-// What the rare paths need of the launch's parameters.
-struct DenseGeo {
-    int N, NR, weff, hoff, log2C, lpl, log2lpl, lp, tp, seg;
-};
-
-// The tile when the kernel's curvature is too small for the screen (bracket
-// search, each row between two rows whose exact argmins are known), or when
-// even the binary64 margin fails (every candidate).  Rare; kept out of line.
-template <typename T, int LAYOUT, typename OFF, int S>
-__device__ __noinline__ int dense_slow(const DenseGeo &p, const T *su, const double *kr64, const unsigned *fx,
-                                       const unsigned *kd, OFF *tt, int mode, int valid)
+// A staged tile whose screen does not hold (a value that is not finite, one
+// line far from the others, or too little curvature for the range): divide and
+// conquer, with its own scale, survivors and margin for every line, and brute
+// force for a line that fails the margin.  Kept out of line, where it leaves the
+// searches' registers alone.
+template <typename T, int LAYOUT, typename OFF>
+__device__ __noinline__ void dense_leave(const PassParams &p, long long tile)
 {
-    const int line = threadIdx.x >> p.log2lpl, g = threadIdx.x & (p.lpl - 1);
-    const int N = p.N, NR = p.NR, weff = p.weff;
-    const bool active = line < valid;
-    constexpr unsigned tol = DenseKey<S>::kThr;
-    const int seg = p.seg, s0 = min(g * seg, NR), s1 = min(s0 + seg, NR);
-    OFF *lt = tt + (active ? line : 0) * p.tp;
-    const unsigned *lf = fx + (active ? line : 0) * p.lp;
-    int rescans = 0;
-    if (mode == DENSE_BRUTE) {
-        if (!active) return 0;
-        for (int r = s0; r < s1; ++r) {
-            const DenseRow<T, LAYOUT> row{su, kr64, lf, kd, N, p.hoff, p.log2C, line, r};
-            Key2 best = key2_max();
-            int bt = 0;
-            for (int t = 0; t < weff; ++t) {
-                const Key2 c = row.sum(t);
-                if (key2_less(c, best)) { best = c; bt = t; }
-            }
-            lt[r] = (OFF)bt;
-        }
-        return 0;
-    }
-    if (active && s0 < s1) {
-        const DenseRow<T, LAYOUT> row{su, kr64, lf + s0, kd, N, p.hoff, p.log2C, line, s0};
-        lt[s0] = (OFF)row.search(0, weff - 1, tol, rescans);
-    }
+    clear_line_ranges(p, reinterpret_cast<LineInfo *>(pass_smem() + p.off_misc + 16));
     __syncthreads();
-    if (!active || s0 >= s1) return rescans;
-    const int jr = (s1 < NR) ? s1 + lt[s1] : N + lt[0];
-    int step = 1;
-    while (2 * step < seg) step *= 2;
-    for (; step; step >>= 1)
-        for (int r = s0 + step; r < s1; r += 2 * step) {
-            const int jl = (r - step) + lt[r - step];
-            const int jh = (r + step < s1) ? r + step + lt[r + step] : jr;
-            const int lo = max(jl - r, 0), hi = min(jh - r, weff - 1);
-            const DenseRow<T, LAYOUT> row{su, kr64, lf + r, kd, N, p.hoff, p.log2C, line, r};
-            lt[r] = (OFF)(lo > hi ? row.search(0, weff - 1, tol, rescans) : row.search(lo, hi, tol, rescans));
-        }
-    return rescans;
+    search_tile<T, LAYOUT, KALGO_MONGE, OFF>(p, tile);
 }
 
 template <typename T, int LAYOUT, typename OFF, int S>
@@ -378,7 +308,6 @@ __device__ __forceinline__ void dense_tile(const CUtensorMap *tmap, const PassPa
     if (!stage_tile<T, LAYOUT>(tmap, p, tile, su, kr64, reinterpret_cast<uint64_t *>(smem + p.off_misc))) return;
 
     const int cl = tid >> p.log2lpl, sub = tid & (lpl - 1);
-    int mode;
     {
         // ---- range of the tile
         const int l = (LAYOUT == LAYOUT_CONTIG) ? cl : tid & (C - 1);
@@ -412,65 +341,56 @@ __device__ __forceinline__ void dense_tile(const CUtensorMap *tmap, const PassPa
         // ---- the tile's scale
         if (tid == 0) dense_scale(key_hi<T>(info->kmin), key_hi<T>(info->kmax), p.kmax, p.curv, Key::kCurv, info);
         __syncthreads();
-        mode = info->mode;
-        const int q = info->q;
-        if (mode != DENSE_BANDS) {
-            // brackets need the binary64 margin; without it, every candidate
-            const double umin = key_bound<T>(info->kmin, true), umax = key_bound<T>(info->kmax, false);
-            const double cmax = __dadd_ru(fmax(fabs(umin), fabs(umax)), p.kmax);
-            if (!isfinite(umax - umin) || !isfinite(cmax) || q > 900 || !(p.curv > __dmul_ru(cmax, 0x1p-49)))
-                mode = DENSE_BRUTE;
+        if (!info->ok) {
+            __syncthreads();                         // everyone has looked
+            const PassParams left = p;
+            dense_leave<T, LAYOUT, OFF>(left, tile);
+            return;
         }
+        const int q = info->q;
         // ---- keys: the halo (its first weff entries repeat one period later:
         // row N, row 0's image, is searched with the last segment when that is
         // a wide one, over its whole window; a few more entries are read by full
         // bands, beside no displacement of the window) and the table
-        if (mode != DENSE_BRUTE) {
-            const double magic = key_magic(q);
-            const unsigned fref = info->fref, kref = info->kref;
-            const int dup = weff;
-            if (mine) {
-                const T *x = (LAYOUT == LAYOUT_CONTIG) ? su + l * N + first : su + tid;
-                const int xs = (LAYOUT == LAYOUT_CONTIG) ? lpl : nthr;
-                unsigned *lfx = fx + l * p.lp, *lfn = lfx + N;
-                auto put = [&](T v, int pos, bool add) {
-                    const unsigned f = ((add ? fixkey(widen(v), magic) : fixshift(widen(v), q)) - fref) & ~Key::kMask;
-                    const int y = pos - p.hoff;                      // in (-N, N)
-                    const int jj = (int)min((unsigned)y, (unsigned)(y + N));
-                    lfx[jj] = f;
-                    if (jj < dup) lfn[jj] = f;
-                };
-                int pos = first;
-                for (; pos + 3 * step < N; pos += 4 * step) {
-                    T v[4];
+        const double magic = key_magic(q);
+        const unsigned fref = info->fref, kref = info->kref;
+        const int dup = weff;
+        if (mine) {
+            const T *x = (LAYOUT == LAYOUT_CONTIG) ? su + l * N + first : su + tid;
+            const int xs = (LAYOUT == LAYOUT_CONTIG) ? lpl : nthr;
+            unsigned *lfx = fx + l * p.lp, *lfn = lfx + N;
+            auto put = [&](T v, int pos, bool add) {
+                const unsigned f = ((add ? fixkey(widen(v), magic) : fixshift(widen(v), q)) - fref) & ~Key::kMask;
+                const int y = pos - p.hoff;                      // in (-N, N)
+                const int jj = (int)min((unsigned)y, (unsigned)(y + N));
+                lfx[jj] = f;
+                if (jj < dup) lfn[jj] = f;
+            };
+            int pos = first;
+            for (; pos + 3 * step < N; pos += 4 * step) {
+                T v[4];
 #pragma unroll
-                    for (int b = 0; b < 4; ++b) v[b] = x[b * xs];
-                    x += 4 * xs;
+                for (int b = 0; b < 4; ++b) v[b] = x[b * xs];
+                x += 4 * xs;
 #pragma unroll
-                    for (int b = 0; b < 4; ++b) put(v[b], pos + b * step, b & 1);
-                }
-                for (; pos < N; pos += step, x += xs) put(*x, pos, false);
-                for (int i = first; i < kDenseOver - 1; i += step) lfn[dup + i] = 0u;
+                for (int b = 0; b < 4; ++b) put(v[b], pos + b * step, b & 1);
             }
-            for (int i = tid; i < kDenseLow + weff + kDenseHigh; i += nthr) {
-                const int t = i - kDenseLow;
-                unsigned k = kDensePad;
-                if (t >= 0 && t < weff) k = (fixkey(kr64[t], magic) - kref) & ~Key::kMask;
-                kpad[i] = k;
-                if (t >= 0 && t < ((weff + 3) & ~3)) kp[t] = k | ((unsigned)(S == kFlat ? t : t >> 2) & Key::kMask);
-            }
+            for (; pos < N; pos += step, x += xs) put(*x, pos, false);
+            for (int i = first; i < kDenseOver - 1; i += step) lfn[dup + i] = 0u;
+        }
+        for (int i = tid; i < kDenseLow + weff + kDenseHigh; i += nthr) {
+            const int t = i - kDenseLow;
+            unsigned k = kDensePad;
+            if (t >= 0 && t < weff) k = (fixkey(kr64[t], magic) - kref) & ~Key::kMask;
+            kpad[i] = k;
+            if (t >= 0 && t < ((weff + 3) & ~3)) kp[t] = k | ((unsigned)(S == kFlat ? t : t >> 2) & Key::kMask);
         }
         __syncthreads();
     }
     const unsigned *kd = kpad + kDenseLow;
     const int NR = p.rows;
     int rescans = 0;
-    if (mode != DENSE_BANDS) {
-        const DenseGeo geo{N, NR, weff, p.hoff, p.log2C, lpl, p.log2lpl, p.lp, p.tp, p.seg};
-        rescans = dense_slow<T, LAYOUT, OFF, S>(geo, su, kr64, fx, kd, tt, mode, tl.valid);
-        if (mode == DENSE_BRUTE && tid == 0) atomicAdd(&p.counters[CNT_FALLBACK], (unsigned long long)tl.valid);
-        __syncthreads();
-    } else if (member) {
+    if (member) {
         auto gsync = [&] {
             if (gsize == 32) __syncwarp();
             else asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "r"(gsize) : "memory");

@@ -744,6 +744,13 @@ __device__ __forceinline__ bool stage_tile(const CUtensorMap *tmap, const PassPa
     return stage_wait(p, bar, 0);
 }
 
+// The dynamic shared memory of the pass kernels.
+__device__ __forceinline__ unsigned char *pass_smem()
+{
+    extern __shared__ __align__(128) unsigned char smem[];
+    return smem;
+}
+
 // Per-line facts of the fixed-point screen, in shared memory.
 struct LineInfo {
     unsigned fref;                  // fixq32(lower bound of u, q)
@@ -755,33 +762,30 @@ struct LineInfo {
     int pad;
 };
 
-// One tile of one axis pass (everything a CTA does).  `tmap` is the 3D TMA
-// descriptor of the source for strided lines (unused otherwise).  OFF holds
-// the rows' argmin offsets in shared memory: bytes when the window has at
-// most 256 displacements (more lines per SM), else 16-bit words.
-template <typename T, int LAYOUT, int ALGO, typename OFF = unsigned short>
-__device__ __forceinline__ void pass_tile(const CUtensorMap *tmap, const PassParams &p, long long tile)
+// Before a tile's per-line ranges are taken; a barrier follows.
+__device__ __forceinline__ void clear_line_ranges(const PassParams &p, LineInfo *li)
 {
-    extern __shared__ __align__(128) unsigned char smem[];
+    if (threadIdx.x < p.C) {
+        li[threadIdx.x].kmin = 0x7fffffff;
+        li[threadIdx.x].kmax = (int)0x80000000;
+    }
+}
+
+// Search and write-back of a staged tile.
+template <typename T, int LAYOUT, int ALGO, typename OFF>
+__device__ __forceinline__ void search_tile(const PassParams &p, long long tile)
+{
+    unsigned char *smem = pass_smem();
     T *su = reinterpret_cast<T *>(smem + p.off_u);
     int *fx = reinterpret_cast<int *>(smem + p.off_fx);
     int *kfx = reinterpret_cast<int *>(smem + p.off_kfx);
     OFF *tt = reinterpret_cast<OFF *>(smem + p.off_t);
     double *kr64 = reinterpret_cast<double *>(smem + p.off_k64);
-    uint64_t *bar = reinterpret_cast<uint64_t *>(smem + p.off_misc);
     LineInfo *li = reinterpret_cast<LineInfo *>(smem + p.off_misc + 16);         // [C]
 
     const int tid = threadIdx.x, nthr = blockDim.x;
     const int N = (int)p.N, C = p.C, weff = p.weff;
     const Tile<LAYOUT> tl = tile_of<LAYOUT>(p, tile);
-
-    // ---- stage the tile
-    if (ALGO == KALGO_MONGE && tid < C) {
-        li[tid].kmin = 0x7fffffff;
-        li[tid].kmax = (int)0x80000000;
-    }
-    if (!stage_tile<T, LAYOUT>(tmap, p, tile, su, kr64, bar)) return;
-
     const int lane = tid & 31, warp = tid >> 5;
 
     if (ALGO == KALGO_MONGE) {
@@ -1111,6 +1115,25 @@ __device__ __forceinline__ void pass_tile(const CUtensorMap *tmap, const PassPar
     count_edges(p, edges);
 }
 
+// One tile of one axis pass (everything a CTA does).  `tmap` is the 3D TMA
+// descriptor of the source for strided lines (unused otherwise).  OFF holds
+// the rows' argmin offsets in shared memory: bytes when the window has at
+// most 256 displacements (more lines per SM), else 16-bit words.
+template <typename T, int LAYOUT, int ALGO, typename OFF = unsigned short>
+__device__ __forceinline__ void pass_tile(const CUtensorMap *tmap, const PassParams &p, long long tile)
+{
+    unsigned char *smem = pass_smem();
+    if (ALGO == KALGO_MONGE) clear_line_ranges(p, reinterpret_cast<LineInfo *>(smem + p.off_misc + 16));
+    if (!stage_tile<T, LAYOUT>(tmap, p, tile, reinterpret_cast<T *>(smem + p.off_u),
+                               reinterpret_cast<double *>(smem + p.off_k64),
+                               reinterpret_cast<uint64_t *>(smem + p.off_misc)))
+        return;
+    search_tile<T, LAYOUT, ALGO, OFF>(p, tile);
+}
+
+// (brute force on strided lines, a warp a row, hides latency by warps alone: 32
+// registers, 2048 threads an SM; 300 x 12000 grid, 5 displacements along the
+// strided axis and 1601 along the other: 742 us a step at 58 registers, 690)
 template <typename T, int LAYOUT, int ALGO, typename OFF>
 __global__ void __launch_bounds__(1024) pass_kernel(const __grid_constant__ CUtensorMap tmap, PassParams p)
 {

@@ -191,6 +191,8 @@ static void layout_smem(AxisPlan &ax, int esize, int algo)
         ax.off_q = (int)off;
         ax.qcap = std::max(31, (int)(group / ax.lpl * ax.N / (ax.dense == kWide ? 2 : 8)));
         off = align_up(off + (size_t)groups * (ax.qcap + 1) * 4, 16);
+        // tiles it leaves to divide and conquer: a table per line in their place
+        off = std::max(off, align_up(ax.off_kfx + (size_t)C * ax.weff * 4, 16));
     }
     ax.off_t = (int)off;
     off = align_up(off + (size_t)C * ax.tp * (ax.t8 ? 1 : 2), 16);
@@ -458,7 +460,7 @@ static hjlo_status shape_lines(AxisPlan &ax, int esize, int algo, int num_sms, s
         ax.log2lpl = ilog2(ax.lpl);
         ax.seg = odd_at_least((NR + ax.lpl - 1) / ax.lpl);
         if (ax.dense != kFlat) ax.seg = ax.dense;
-        ax.gs = 1;
+        ax.gs = pivot_group(ax.weff, ax.seg, ax.lpl, nullptr);   // (tiles left to divide and conquer)
         ax.t8 = 0;
         ax.tp = (int)N;
         while (ax.tp % 4 != 2) ++ax.tp;

@@ -6,14 +6,6 @@
 
 namespace hjlo {
 
-// The dynamic shared memory of the pass kernels.
-__device__ __forceinline__ unsigned char *pass_smem()
-{
-    extern __shared__ __align__(128) unsigned char smem[];
-    return smem;
-}
-
-
 // One work item of the persistent batched pass: tiles [tile0, tile0 + ntile)
 // of instance `inst` on axis `axis`, launch shape `shape` (a (group, axis)
 // entry of PersistParams::shapes).

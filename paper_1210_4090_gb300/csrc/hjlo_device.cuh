@@ -371,18 +371,38 @@ __device__ __forceinline__ int wrapN(int x, int N)
     return (x >= N) ? x - N : x;
 }
 
-// Exact scan of halo indices [lo, hi] for row r: smallest key, ascending jj.
+// Exact scan of halo indices [lo, hi] for row r: smallest key, smallest jj.
+// Four running minima, as one chain of compares and selects is what a lane
+// would wait for.
 template <typename T, int LAYOUT>
 __device__ __forceinline__ void exact_scan(const PassParams &p, const T *su, const double *kr64, int l, int r,
                                            int lo, int hi, Key2 &best, int &bt)
 {
     const int N = (int)p.N;
     int pos = wrapN(lo + p.hoff, N);
-    for (int jj = lo; jj <= hi; ++jj) {
-        const Key2 key = key2(__dadd_rn(widen(su[uidx<LAYOUT>(p, l, pos)]), kr64[jj - r]));
-        if (key2_less(key, best)) { best = key; bt = jj - r; }
-        pos = (pos + 1 == N) ? 0 : pos + 1;
+    Key2 kb[4];
+    int jb[4];
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+        kb[b] = key2_max();
+        jb[b] = lo;
     }
+    for (int jj = lo; jj <= hi; jj += 4)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            const int j = min(jj + b, hi);
+            const Key2 key = key2(__dadd_rn(widen(su[uidx<LAYOUT>(p, l, pos)]), kr64[j - r]));
+            const bool less = key2_less(key, kb[b]);
+            kb[b] = less ? key : kb[b];
+            jb[b] = less ? j : jb[b];
+            if (jj + b < hi) pos = (pos + 1 == N) ? 0 : pos + 1;
+        }
+#pragma unroll
+    for (int b = 0; b < 4; ++b)
+        if (key2_less(kb[b], best) || (key2_eq(kb[b], best) && jb[b] - r < bt)) {
+            best = kb[b];
+            bt = jb[b] - r;
+        }
 }
 
 // Screened search of row r over the offsets t in [tlo, thi] (halo index
@@ -909,15 +929,21 @@ __device__ __forceinline__ void search_tile(const PassParams &p, long long tile)
         const int s0 = min(g * S, NR), s1 = min((g + 1) * S, NR);
         const int o = g & (GS - 1);
         const int rp = min((g - o) * S, NR);  // the group's pivot row
-        if (active && fallback) {
-            // brute force over each lane's own segment of rows
-            for (int r = s0; r < s1; ++r) {
-                Key2 best = key2_max();
-                int bt = 0;
-                exact_scan<T, LAYOUT>(p, su, kr64, line, r, r, r + weff - 1, best, bt);
-                lt[r] = (OFF)bt;
+        {
+            // brute force, a line's lanes on neighbouring rows (written back after
+            // a barrier); wide strided tiles line index fastest, so that a warp's
+            // words are adjacent (a line's are C apart, in 16 / C banks)
+            const bool byline = LAYOUT == LAYOUT_CONTIG || C < 8;
+            const int l = byline ? line : tid & (C - 1), step = byline ? p.lpl : nthr >> p.log2C;
+            if (l < tl.valid && li[l].fallback) {
+                for (int r = byline ? g : tid >> p.log2C; r < NR; r += step) {
+                    Key2 best = key2_max();
+                    int bt = 0;
+                    exact_scan<T, LAYOUT>(p, su, kr64, l, r, r, r + weff - 1, best, bt);
+                    tt[l * p.tp + r] = (OFF)bt;
+                }
             }
-            if (g == 0) atomicAdd(&p.counters[CNT_FALLBACK], 1ull);
+            if (active && fallback && g == 0) atomicAdd(&p.counters[CNT_FALLBACK], 1ull);
         }
         if (GS == 1) {
             // P1: every segment's first row scans the whole window
@@ -1032,9 +1058,10 @@ __device__ __forceinline__ void search_tile(const PassParams &p, long long tile)
         }
         if (LAYOUT == LAYOUT_CONTIG) {
             // Every row's argmin was found by a lane of the warp that owns the
-            // row's segment (divide and conquer, offload and fallback lines all
-            // stay inside the warp after P2), so each warp writes its own rows
-            // back as soon as it is done: no block barrier, coalesced stores.
+            // row's segment (divide and conquer and offload stay inside the
+            // warp after P2) or before P1's barrier (brute force), so each warp
+            // writes its own rows back as soon as it is done: no block barrier,
+            // coalesced stores.
             __syncwarp();
             pdl_next();
             const int nl = (lpl >= 32) ? 1 : (32 >> p.log2lpl);     // lines held by this warp

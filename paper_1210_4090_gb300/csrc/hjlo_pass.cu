@@ -275,10 +275,19 @@ static int dense_segment(const AxisPlan &ax, long long NR, long long nlines, int
     if (!holds(lpl, wide ? kWide : 13) || (long long)lpl * cmin > dense_threads(13) || lpl > ax.N || (wide && lpl < 32))
         return 0;
     // few lanes in all: a pivot's scan of the window, done by one lane, would be
-    // most of the launch (8192-point line, 291 displacements, 15 blocks: 15 us
-    // a pass against 11.7 by divide and conquer, which shares it; 32768 points,
-    // 581 displacements, 57 blocks of 64 lanes: 15.6 against 14.4)
-    if (!hinted && nlines * lpl < (wide ? 32LL : 64LL) * num_sms) return 0;
+    // most of the launch, which divide and conquer shares.  9 or 13 rows a
+    // segment, one line, 64 lanes a block: 65536 points, 291 displacements 15.3
+    // us a pass against 14.3, 100000 points 18.0 against 13.9; 320 x 320 grid,
+    // 129 displacements, 32 lanes a line 22.3 against 20.8; but 128 lanes: 1000 x
+    // 100 grid, 101 displacements 36 against 39.5, and from 481 displacements on
+    // its shared scan meets bank conflicts (80000 points, 501 displacements 18.9
+    // against 28.5).  11 rows: 50000 points, 601 displacements, 84 blocks of 64
+    // lanes 22.4 against 19.2, 801 displacements 24.9 against 34.1.
+    const long long few = wide ? 32 : lpl < 128 && ax.weff <= 480 ? 100 : 64;
+    if (!hinted && nlines * lpl < few * num_sms) return 0;
+    // four warps at least, for staging and keys and for lines left to brute force
+    // (one line of 65536 points, 521 displacements: 64 lanes 21.2 us, 128 20.1)
+    if (wide && !hinted) lpl = std::max(lpl, 128);
     *lanes = lpl;
     if (wide) return kWide;
     return holds(lpl, 9) && lpl * cmin <= dense_threads(9) ? 9 : 13;

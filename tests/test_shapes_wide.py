@@ -53,3 +53,18 @@ def test_block_rows(N, weff, rows, seg):
     if seg:
         assert s["segment_rows"] == seg, s
     assert s["threads"] >= (128 if weff > 512 else 32), s
+
+
+@pytest.mark.parametrize("N,lines,weff,seg", [
+    (65536, 1, 291, 0), (80000, 1, 201, 0), (320, 320, 129, 0),   # 64 and 32 lanes a line: divide and conquer
+    (80000, 1, 501, 9), (180000, 1, 201, 13), (1 << 18, 1, 201, 9), (448, 448, 129, 9)])
+def test_few_lanes_go_to_divide_and_conquer(N, lines, weff, seg):
+    s = hjlo.shape_query(N, lines, weff)
+    assert (s["segment_rows"] == seg) if seg else s["segment_rows"] < 9, s
+    assert s["threads"] >= 64, s
+
+
+def test_wide_windows_have_four_warps():
+    for N, weff in [(65536, 521), (50000, 601), (100000, 601)]:
+        s = hjlo.shape_query(N, 1, weff)
+        assert s["segment_rows"] == 11 and s["threads"] >= 128, (N, weff, s)

@@ -753,7 +753,7 @@ __device__ __forceinline__ void dense_tile(const CUtensorMap *tmap, const PassPa
         }
     } else {
         __syncthreads();
-        edges = write_rows_strided<T, OFF>(p, tl, su, tt, kr64);
+        edges = write_rows_strided<T, OFF, 4>(p, tl, su, tt, kr64);
     }
     count_edges(p, edges);
 }

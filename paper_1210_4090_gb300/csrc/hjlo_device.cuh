@@ -562,10 +562,10 @@ __device__ __forceinline__ void count_edges(const PassParams &p, int edges)
 // the grid is row i0's, xs elements on to the next): the exact value
 // fl(u[src] + k[d]) at the recorded argmin, minus fl(h V) when the pass
 // carries the potential term (HV), stored (binary32: rounded), with the
-// optional argmin (AM).  Four rows per thread at a time, their loads issued
+// optional argmin (AM).  B rows per thread at a time, their loads issued
 // together; the source's position wraps by an unsigned minimum.  Returns how
 // many of the rows' argmins sit on a partial window's edge.
-template <typename T, typename OFF, bool HV, bool AM>
+template <typename T, typename OFF, int B, bool HV, bool AM>
 __device__ __forceinline__ int write_rows(const PassParams &p, const T *lu, int sh, const OFF *lt, const double *kr64,
                                           int i0, int i1, int step, long long x0, long long xs)
 {
@@ -587,29 +587,29 @@ __device__ __forceinline__ int write_rows(const PassParams &p, const T *lu, int 
         return (int)min((unsigned)hh, (unsigned)(hh - N));
     };
     int i = i0;
-    for (; i + 3 * step < i1; i += 4 * step) {
-        double hvb[4], m[4];
-        int t[4];
+    for (; B > 1 && i + (B - 1) * step < i1; i += B * step) {
+        double hvb[B], m[B];
+        int t[B];
 #pragma unroll
-        for (int b = 0; b < 4; ++b) {
+        for (int b = 0; b < B; ++b) {
             if (HV) hvb[b] = __ldg(gh + b * xs);
             t[b] = lt[i + b * step];
         }
 #pragma unroll
-        for (int b = 0; b < 4; ++b) {
+        for (int b = 0; b < B; ++b) {
             m[b] = one(t[b], h);
             h = next(h);
             edges += on_edge(t[b], weff);
         }
 #pragma unroll
-        for (int b = 0; b < 4; ++b) {
+        for (int b = 0; b < B; ++b) {
             if (HV) m[b] = __dsub_rn(m[b], p.hv_scaled ? __dmul_rn(p.hscale, hvb[b]) : hvb[b]);
             store_val(gd + b * xs, m[b]);
             if (AM) ga[b * xs] = p.dhi - t[b];
         }
-        gd += 4 * xs;
-        if (HV) gh += 4 * xs;
-        if (AM) ga += 4 * xs;
+        gd += B * xs;
+        if (HV) gh += B * xs;
+        if (AM) ga += B * xs;
     }
     for (; i < i1; i += step) {
         const int t = lt[i];
@@ -626,15 +626,15 @@ __device__ __forceinline__ int write_rows(const PassParams &p, const T *lu, int 
     return p.edge ? edges : 0;
 }
 
-template <typename T, typename OFF>
+template <typename T, typename OFF, int B>
 __device__ __forceinline__ int write_rows(const PassParams &p, const T *lu, int sh, const OFF *lt, const double *kr64,
                                           int i0, int i1, int step, long long x0, long long xs)
 {
     if (p.amin)
-        return p.hv ? write_rows<T, OFF, true, true>(p, lu, sh, lt, kr64, i0, i1, step, x0, xs)
-                    : write_rows<T, OFF, false, true>(p, lu, sh, lt, kr64, i0, i1, step, x0, xs);
-    return p.hv ? write_rows<T, OFF, true, false>(p, lu, sh, lt, kr64, i0, i1, step, x0, xs)
-                : write_rows<T, OFF, false, false>(p, lu, sh, lt, kr64, i0, i1, step, x0, xs);
+        return p.hv ? write_rows<T, OFF, B, true, true>(p, lu, sh, lt, kr64, i0, i1, step, x0, xs)
+                    : write_rows<T, OFF, B, false, true>(p, lu, sh, lt, kr64, i0, i1, step, x0, xs);
+    return p.hv ? write_rows<T, OFF, B, true, false>(p, lu, sh, lt, kr64, i0, i1, step, x0, xs)
+                : write_rows<T, OFF, B, false, false>(p, lu, sh, lt, kr64, i0, i1, step, x0, xs);
 }
 
 // Rows i0, i0 + step, ... < i1 of a contiguous line whose row 0 is element xb.
@@ -642,17 +642,17 @@ template <typename T, typename OFF>
 __device__ __forceinline__ int write_rows_contig(const PassParams &p, const T *lu, const OFF *lt, const double *kr64,
                                                  long long xb, int i0, int i1, int step)
 {
-    return write_rows<T, OFF>(p, lu, 0, lt, kr64, i0, i1, step, xb + i0, step);
+    return write_rows<T, OFF, 4>(p, lu, 0, lt, kr64, i0, i1, step, xb + i0, step);
 }
 
 // A tile of strided lines (line index fastest).
-template <typename T, typename OFF>
+template <typename T, typename OFF, int B>
 __device__ __forceinline__ int write_rows_strided(const PassParams &p, const Tile<LAYOUT_STRIDED> &tl, const T *su,
                                                   const OFF *tt, const double *kr64)
 {
     const int l = threadIdx.x & (p.C - 1), i0 = threadIdx.x >> p.log2C, step = blockDim.x >> p.log2C;
     if (l >= tl.valid) return 0;
-    return write_rows<T, OFF>(p, su + l, p.log2C, tt + l * p.tp, kr64, i0, (int)p.N, step,
+    return write_rows<T, OFF, B>(p, su + l, p.log2C, tt + l * p.tp, kr64, i0, (int)p.N, step,
                               tl.base + l + (long long)i0 * tl.pstride, (long long)step * tl.pstride);
 }
 
@@ -1146,7 +1146,7 @@ __device__ __forceinline__ void search_tile(const PassParams &p, long long tile)
             edges = write_rows_contig<T, OFF>(p, su + l * N, tt + l * p.tp, kr64, xb, sub, rows, lanes);
         }
     } else {
-        edges = write_rows_strided<T, OFF>(p, tl, su, tt, kr64);
+        edges = write_rows_strided<T, OFF, ALGO == KALGO_BRUTE ? 1 : 4>(p, tl, su, tt, kr64);
     }
     count_edges(p, edges);
 }
@@ -1171,7 +1171,7 @@ __device__ __forceinline__ void pass_tile(const CUtensorMap *tmap, const PassPar
 // registers, 2048 threads an SM; 300 x 12000 grid, 5 displacements along the
 // strided axis and 1601 along the other: 742 us a step at 58 registers, 690)
 template <typename T, int LAYOUT, int ALGO, typename OFF>
-__global__ void __launch_bounds__(1024) pass_kernel(const __grid_constant__ CUtensorMap tmap, PassParams p)
+__global__ void __launch_bounds__(1024, LAYOUT == LAYOUT_STRIDED && ALGO == KALGO_BRUTE ? 2 : 1) pass_kernel(const __grid_constant__ CUtensorMap tmap, PassParams p)
 {
     const long long tile = blockIdx.x;
     if (tile >= p.ntiles) return;

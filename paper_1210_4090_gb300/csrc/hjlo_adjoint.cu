@@ -307,7 +307,8 @@ hjlo_status launch_adjoint_pass(const AxisPlan &ax, double dx, double *ub, const
     p.weff = ax.weff;
     p.off_g = sh.off_g;
     p.dx = dx;
-    cudaError_t e = launch_pdl(sh.layout == LAYOUT_CONTIG ? adjoint_pass_kernel<LAYOUT_CONTIG>
+    cudaError_t e = launch_pdl(true,
+                               sh.layout == LAYOUT_CONTIG ? adjoint_pass_kernel<LAYOUT_CONTIG>
                                                           : adjoint_pass_kernel<LAYOUT_STRIDED>,
                                (unsigned)sh.ntiles, sh.threads, sh.smem, st, p);
     if (e != cudaSuccess) return cuda_error(e, "adjoint pass launch");

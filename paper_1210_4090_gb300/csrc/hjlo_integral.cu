@@ -356,7 +356,7 @@ hjlo_status hjlo_integral_run(hjlo_integral *s, double *u, int64_t nsteps)
     const unsigned blocks = (unsigned)((s->npts * kIntegralSplit + 255) / 256);
     for (long long n = 0; n < nsteps; ++n) {
         if (s->d_hS)
-            e = launch_pdl(integral_table_kernel, (unsigned)((s->npts + 31) / 32), 32 * kCostParts, 0, s->stream, a, b,
+            e = launch_pdl(true, integral_table_kernel, (unsigned)((s->npts + 31) / 32), 32 * kCostParts, 0, s->stream, a, b,
                            s->d_hS, s->d_K, s->d_disp, (int)s->ndisp, (int)s->shape[0], (int)s->shape[1],
                            (int)s->shape[2], s->npts);
         else

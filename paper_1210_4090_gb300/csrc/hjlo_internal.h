@@ -59,10 +59,14 @@ struct AxisPlan {
 // it may start before they end: 1-2 us of each launch of a chain of small ones
 // (gradients on 512^2, 128 steps: 8.8 -> 7.7 ms; 8192-point line, 289 steps:
 // 3.3 -> 2.6; decomposition of 2^18 points, five launches a pass: 74 -> 70.6).
-// Of the larger grids 90x121x135 gains 10 %, 256^3 2 %, and
-// 701 x 1013 loses 6 %.
+// Of the larger grids 90x121x135 gains 10 %, 256^3 2 %.  A launch whose CTAs
+// wait gathers them on the SMs that are free first, which costs passes bound by
+// the binary64 pipe more than it gives: 65536-point line, 201 displacements, brute
+// force 58 us a pass with it, 46 without; 1000 x 1000 grid, 5 displacements,
+// binary32 532 and 451 a step.
 template <typename... P, typename... A>
-cudaError_t launch_pdl(void (*kernel)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t st, A &&...args)
+cudaError_t launch_pdl(bool early, void (*kernel)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t st,
+                       A &&...args)
 {
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -73,7 +77,7 @@ cudaError_t launch_pdl(void (*kernel)(P...), unsigned grid, unsigned threads, si
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = early ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 

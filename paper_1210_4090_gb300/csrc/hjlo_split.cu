@@ -1032,14 +1032,14 @@ hjlo_status launch_split(const AxisPlan &ax, const void *src, void *dst, const d
     const long long chunks = p.lines * p.B;
     const size_t stage = sizeof(int) * 3 * (size_t)(p.Wl + p.B);
     const bool staged = stage <= kStitchStage;
-    cudaError_t e = launch_pdl(split_classify, (unsigned)chunks, kSplitThreads, 0, st, p);
+    cudaError_t e = launch_pdl(true, split_classify, (unsigned)chunks, kSplitThreads, 0, st, p);
     if (e == cudaSuccess)
-        e = launch_pdl(split_local_cut, (unsigned)((chunks + kCutWarps - 1) / kCutWarps), 32 * kCutWarps, 0, st, p);
+        e = launch_pdl(true, split_local_cut, (unsigned)((chunks + kCutWarps - 1) / kCutWarps), 32 * kCutWarps, 0, st, p);
     if (e == cudaSuccess)
-        e = launch_pdl(split_stitch, (unsigned)p.lines, kStitchThreads, staged ? stage : 0, st, p, staged ? 1 : 0);
-    if (e == cudaSuccess) e = launch_pdl(split_pieces, (unsigned)chunks, kSplitThreads, 0, st, p);
+        e = launch_pdl(true, split_stitch, (unsigned)p.lines, kStitchThreads, staged ? stage : 0, st, p, staged ? 1 : 0);
+    if (e == cudaSuccess) e = launch_pdl(true, split_pieces, (unsigned)chunks, kSplitThreads, 0, st, p);
     if (e == cudaSuccess)
-        e = launch_pdl(split_emit, (unsigned)(p.lines * p.nblk * (p.share ? 2 : 1)), kEmitThreads, ax.smem, st, p);
+        e = launch_pdl(true, split_emit, (unsigned)(p.lines * p.nblk * (p.share ? 2 : 1)), kEmitThreads, ax.smem, st, p);
     if (e != cudaSuccess) return cuda_error(e, "decomposition kernel launch");
     return HJLO_OK;
 }

@@ -592,7 +592,7 @@ __device__ __forceinline__ int write_rows(const PassParams &p, const T *lu, int 
         int t[B];
 #pragma unroll
         for (int b = 0; b < B; ++b) {
-            if (HV) hvb[b] = __ldg(gh + b * xs);
+            if (HV) hvb[b] = gh[b * xs];
             t[b] = lt[i + b * step];
         }
 #pragma unroll

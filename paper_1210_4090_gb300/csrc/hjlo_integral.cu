@@ -141,9 +141,11 @@ constexpr int kCostParts = 8;          // warps that share 32 outputs
 // rows are read whole), a block's warps share the displacements.  Candidates are
 // compared as order-preserving 32-bit pairs, which leaves the binary64 pipe to
 // the add and the subtract; a NaN never wins, as with a binary64 comparison.
+// (src, dst and hS without __restrict__ or __ldg: the kernel is resident while
+// the one before it still writes them.)
 __global__ void __launch_bounds__(32 * kCostParts) integral_table_kernel(
-    const double *__restrict__ src, double *__restrict__ dst, const double *__restrict__ hS,
-    const double *__restrict__ K, const int *__restrict__ disp, int ndisp, int n0, int n1, int n2, long long npts)
+    const double *src, double *dst, const double *hS, const double *__restrict__ K, const int *__restrict__ disp,
+    int ndisp, int n0, int n1, int n2, long long npts)
 {
     __shared__ double part[kCostParts][32];
     pdl_wait();
@@ -163,7 +165,7 @@ __global__ void __launch_bounds__(32 * kCostParts) integral_table_kernel(
             y1 += (y1 < 0) ? n1 : 0;
             y2 += (y2 < 0) ? n2 : 0;
             const long long y = ((long long)y0 * n1 + y1) * n2 + y2;
-            const double c = __dsub_rn(__dadd_rn(src[y], __ldg(K + di)), __ldg(hS + di * npts + y));
+            const double c = __dsub_rn(__dadd_rn(src[y], __ldg(K + di)), hS[di * npts + y]);
             const dkey_pair ck = dkey_of(c);
             if (key2_less(ck, bk)) {
                 bk = ck;

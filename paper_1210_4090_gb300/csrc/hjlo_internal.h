@@ -56,7 +56,10 @@ struct AxisPlan {
 };
 
 // Launches a kernel that waits for its predecessors itself (pdl_wait), so that
-// it may start before they end: 1-2 us of each launch of a chain of small ones
+// it may start before they end.  The state, the potential and whatever else a
+// kernel before it may have written is then not read-only while it is resident:
+// no __restrict__ and no read-only load (__ldg) on those.  An early start is worth
+// 1-2 us of each launch of a chain of small ones
 // (gradients on 512^2, 128 steps: 8.8 -> 7.7 ms; 8192-point line, 289 steps:
 // 3.3 -> 2.6; decomposition of 2^18 points, five launches a pass: 74 -> 70.6).
 // Of the larger grids 90x121x135 gains 10 %, 256^3 2 %.  A launch whose CTAs

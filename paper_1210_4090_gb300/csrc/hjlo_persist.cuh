@@ -130,6 +130,9 @@ __global__ void __launch_bounds__(1024) pass_kernel_persist(const __grid_constan
                     persist_tile<T, LAYOUT_CONTIG>(&bi->tmap, s_p, it.tile0 + t);
                 else
                     persist_tile<T, LAYOUT_STRIDED>(&bi->tmap, s_p, it.tile0 + t);
+                // this tile's reads and plain stores of shared memory (generic
+                // proxy) before the next one's bulk copies (async proxy) fill it
+                fence_proxy_async_smem();
                 __syncthreads();
                 if (tid == 0) mbar_inval(reinterpret_cast<uint64_t *>(pass_smem() + s_p.off_misc));
                 __syncthreads();

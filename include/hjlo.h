@@ -215,7 +215,8 @@ hjlo_status hjlo_plan_set_tolerance(hjlo_plan *plan, double eta);
  * Autotune the launch shapes of a plan's monotone passes (no counterpart in
  * the paper: results never depend on the launch shape, only the time does).
  * Axis by axis, shapes around the current one -- lanes per line and lines
- * per tile halved / kept / doubled, wide-bracket offload on / off, and for
+ * per tile halved / kept / doubled, wide-bracket offload on / off (divide and
+ * conquer; the register-tile searches have none and are tried once), and for
  * an axis in row blocks the rows per block halved / kept / doubled -- are
  * timed with CUDA events on nsteps steps from a device copy of u (u itself
  * is not modified; V: npts binary64 or NULL), and each axis keeps the

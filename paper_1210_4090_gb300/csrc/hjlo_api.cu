@@ -591,6 +591,7 @@ hjlo_status hjlo_plan_autotune(hjlo_plan *p, const void *u, const double *V, int
             if (t.lpl == best.lpl && t.C == best.C && t.wide_mul == best.wide_mul && t.wide_add == best.wide_add &&
                 t.vR == best.vR)
                 continue;
+            if (t.dense && h.wide_mul == 0) continue;        // no offload there: the same launch again
             AxisPlan keep = p->ax[a];
             p->ax[a] = t;
             float ms = 0.0f;

@@ -712,6 +712,7 @@ hjlo_status hjlo_batch_autotune(hjlo_batch *b, const void *const *u, const doubl
                     continue;
                 if (t.lpl == best.lpl && t.C == best.C && t.wide_mul == best.wide_mul && t.wide_add == best.wide_add)
                     continue;
+                if (t.dense && h.wide_mul == 0) continue;    // no offload there: the same launch again
                 apply_group_shape(b, g, a, t);
                 drop_graphs(b);
                 float ms = 0.0f;

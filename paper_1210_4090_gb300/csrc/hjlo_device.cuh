@@ -91,7 +91,8 @@ struct PassParams {
     // tile line rl * vblocks + b, staged as a periodic line of N = vR + weff - 1
     // points: halo index jj <-> real position (b * vR + jj + vhoff) mod vN.
     // Its first vR rows see no wrap, so their minima are the real rows', and
-    // only they are searched, with row vR as the last segment's right bracket.
+    // only they are searched: the last segment's right bracket is row N,
+    // the periodic image of row 0, a valid bracket for every row of the line.
     long long vN, vblocks;
     int vR, vhoff;
 };
@@ -944,16 +945,6 @@ __device__ __forceinline__ void search_tile(const PassParams &p, long long tile)
             }
             if (active && fallback && g == 0) atomicAdd(&p.counters[CNT_FALLBACK], 1ull);
         }
-        // a row block's row after the last, by its line's last lanes: the right
-        // bracket of its last segment (row 0's image lies a window further on)
-        const bool outer = NR < N;
-        if (outer) {
-            int unused = 0;
-            const bool has = work && g == p.lpl - 1;
-            const int t = row_or_offload<T, LAYOUT>(p, su, fx, kfx, kr64, lsafe, NR, 0, weff - 1, thr_add, has, 0,
-                                                    unused);
-            if (has) lt[NR] = (OFF)t;
-        }
         if (GS == 1) {
             // P1: every segment's first row scans the whole window
             if (work && s0 < s1)
@@ -1020,7 +1011,7 @@ __device__ __forceinline__ void search_tile(const PassParams &p, long long tile)
                 if (has) {
                     const int jl = rp + lt[rp];
                     const int rn = min((g - o + GS) * S, NR);
-                    const int jr = (rn < NR) ? rn + lt[rn] : outer ? NR + lt[NR] : N + lt[0];
+                    const int jr = (rn < NR) ? rn + lt[rn] : N + lt[0];
                     lo = max(jl - s0, 0);
                     hi = min(jr - s0, weff - 1);
                     if (lo > hi) { lo = 0; hi = weff - 1; }   // never for a Monge matrix
@@ -1038,7 +1029,7 @@ __device__ __forceinline__ void search_tile(const PassParams &p, long long tile)
             // every lane walks the block-uniform segment length S (rows past
             // its segment's end are predicated off)
             const bool dc = work && s1 - s0 >= 2;
-            const int jnext = !dc ? 0 : (s1 < NR) ? s1 + lt[s1] : outer ? NR + lt[NR] : N + lt[0];
+            const int jnext = dc ? ((s1 < NR) ? (s1 + lt[s1]) : (N + lt[0])) : 0;
             const int nr = s1 - s0;
             int step = 1;
             while (step * 2 < S) step *= 2;

@@ -232,7 +232,8 @@ static int pivot_group(int weff, int S, int lpl, double *cost)
 }
 
 // The banded search's kind (rows per segment; hjlo_dense.cuh) and its lanes per
-// line, or 0 for divide and conquer.  `cmin`: the fewest lines a tile can hold.
+// line, or 0 for divide and conquer.  `cmin`: the fewest lines a tile can hold;
+// `sparing`: few lanes go to divide and conquer.
 // Flat for windows of up to kFlatMaxWindow: the fewest lanes a line that give
 // every SM 512 threads and a lane four turns of four rows at most, since the
 // more lines a tile then holds, the longer its rows in memory (256^3 grid,
@@ -243,7 +244,7 @@ static int pivot_group(int weff, int S, int lpl, double *cost)
 // leaves at most 30 % of them idle, and a pivot scans the whole window, weff / 9
 // add-minimums and shared-memory words a row, which bounds the windows.
 static int dense_segment(const AxisPlan &ax, long long NR, long long nlines, int cmin, int num_sms,
-                         const ShapeHints &hint, int *lanes)
+                         const ShapeHints &hint, bool sparing, int *lanes)
 {
     if (ax.weff > kDenseMaxWindow) return 0;
     const bool hinted = hint.lpl > 0 && (hint.lpl & (hint.lpl - 1)) == 0 && hint.lpl <= ax.N;
@@ -259,6 +260,11 @@ static int dense_segment(const AxisPlan &ax, long long NR, long long nlines, int
             const double use = (double)quads / (double)(turns * lpl);
             if (use > 1.1 * score || nlines * lpl <= 32LL * num_sms) { score = use; best = lpl; }
         }
+        // (few lanes with long turns: 900 x 60 grid, 91 displacements 25.6 us a step
+        // against 19.9 by divide and conquer; 278 x 36, 31 displacements 27 against 30)
+        if (sparing && !hinted && (quads + best - 1) / best * ax.weff > 128 && quads > best &&
+            nlines * best < 64LL * num_sms)
+            return 0;
         if (hinted && hint.lpl <= most) best = hint.lpl;
         *lanes = best;
         return (quads + best - 1) / best <= 16 ? kFlat : 0;
@@ -281,9 +287,16 @@ static int dense_segment(const AxisPlan &ax, long long NR, long long nlines, int
     // 129 displacements, 32 lanes a line 22.3 against 20.8; but 128 lanes: 1000 x
     // 100 grid, 101 displacements 36 against 39.5, and from 481 displacements on
     // its shared scan meets bank conflicts (80000 points, 501 displacements 18.9
-    // against 28.5).  11 rows: 50000 points, 601 displacements, 84 blocks of 64
-    // lanes 22.4 against 19.2, 801 displacements 24.9 against 34.1.
-    const long long few = wide ? 32 : lpl < 128 && ax.weff <= 480 ? 100 : 64;
+    // against 28.5).  11 rows, whose lanes share the pivots: 16000 points, 601
+    // displacements, 27 blocks 21.3 against 24.1 to 19.1 (as a shock lies in the
+    // groups), 25000 points 25.1 to 21.6 against 21.4 to 18.3, 20000 points, 1201
+    // displacements 29.8 against 45.5, 2001 34.7 against 98.
+    // Contiguous lines with 16 lanes: 1000 x 166 grid, 99 displacements 25.6 us a
+    // step against 22.5, 1500 x 208 grid 30.9 against 26.6, 1000 x 130 21.3 against
+    // 22.1.
+    long long few = ax.inner == 1 && lpl == 16 ? 160 : 100;
+    if (!sparing || lpl >= 128 || ax.weff > 480) few = 64;
+    if (wide) few = ax.weff > 640 ? 0 : 32;
     if (!hinted && nlines * lpl < few * num_sms) return 0;
     // four warps at least, for staging and keys and for lines left to brute force
     // (one line of 65536 points, 521 displacements: 64 lanes 21.2 us, 128 20.1)
@@ -344,7 +357,7 @@ std::vector<ShapeHints> tune_candidates(const AxisPlan &ax)
 }
 
 static hjlo_status shape_lines(AxisPlan &ax, int esize, int algo, int num_sms, size_t smem_optin,
-                               long long replicas, const ShapeHints *hints);
+                               long long replicas, const ShapeHints *hints, bool sparing = true);
 
 // Rows per block for a contiguous axis, or 0 to launch whole lines.  Blocks
 // are used when the window is at most a quarter of the line and either a
@@ -428,8 +441,9 @@ hjlo_status shape_launch(AxisPlan &ax, int esize, int algo, int num_sms, size_t 
 }
 
 static hjlo_status shape_lines(AxisPlan &ax, int esize, int algo, int num_sms, size_t smem_optin,
-                               long long replicas, const ShapeHints *hints)
+                               long long replicas, const ShapeHints *hints, bool sparing)
 {
+    const AxisPlan asked = ax;
     const ShapeHints hint = hints ? *hints : env_hints();
     ax.algo = algo;
     ax.layout = (ax.inner == 1) ? LAYOUT_CONTIG : LAYOUT_STRIDED;
@@ -464,7 +478,8 @@ static hjlo_status shape_lines(AxisPlan &ax, int esize, int algo, int num_sms, s
 
     // rows searched per line (a row block searches only its own rows)
     const long long NR = (ax.rows > 0 && ax.rows < N) ? ax.rows : N;
-    ax.dense = (algo == KALGO_MONGE) ? dense_segment(ax, NR, nlines, cmin, num_sms, hint, &ax.lpl) : 0;
+    ax.dense = (algo == KALGO_MONGE) ? dense_segment(ax, NR, nlines, cmin, num_sms, hint, sparing, &ax.lpl)
+                                     : 0;
     if (ax.dense) {
         ax.log2lpl = ilog2(ax.lpl);
         ax.seg = odd_at_least((NR + ax.lpl - 1) / ax.lpl);
@@ -558,8 +573,15 @@ static hjlo_status shape_lines(AxisPlan &ax, int esize, int algo, int num_sms, s
     ax.C = C;
     layout_smem(ax, esize, algo);
     const long long most = ax.dense ? dense_threads(ax.dense) : 1024;
-    if (ax.smem > smem_optin || (long long)C * lanes > most)
+    if (ax.smem > smem_optin || (long long)C * lanes > most) {
+        // (strided lines: divide and conquer's lanes times the fewest lines of a
+        // tile can pass a CTA's, the register tiles' fewer ones not)
+        if (algo == KALGO_MONGE && !ax.dense && sparing) {
+            ax = asked;
+            return shape_lines(ax, esize, algo, num_sms, smem_optin, replicas, hints, false);
+        }
         return set_error(HJLO_EUNSUPPORTED, "a line of %lld points does not fit in shared memory", N);
+    }
     const size_t budget = std::min<size_t>(110 * 1024, smem_optin);
     const long long cap = (algo == KALGO_MONGE) ? (ax.dense ? 256 : 128) : 512;
     while (2 * C <= std::max(cmax, C) && (long long)2 * C * lanes <= cap &&

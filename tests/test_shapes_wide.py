@@ -45,7 +45,7 @@ def test_long_lines_that_fit_are_whole(N, lines, weff):
 @pytest.mark.parametrize("N,weff,rows,seg", [
     (1 << 18, 3271, 3270, 11), (65536, 1601, 1600, 11),    # weff - 1 rows, searched in segments of 11
     (1 << 18, 201, 1725, 9), (65536, 291, 432, None),      # one SM's share; few lanes: divide and conquer
-    (20000, 2401, 4800, None), (1 << 18, 3801, 7600, None),      # divide and conquer: 2 (weff - 1) rows
+    (20000, 2401, 2400, 11), (1 << 18, 3801, 7600, None),      # divide and conquer: 2 (weff - 1) rows
     (8192, 291, 290, None)])
 def test_block_rows(N, weff, rows, seg):
     s = hjlo.shape_query(N, 1, weff)
@@ -68,3 +68,9 @@ def test_wide_windows_have_four_warps():
     for N, weff in [(65536, 521), (50000, 601), (100000, 601)]:
         s = hjlo.shape_query(N, 1, weff)
         assert s["segment_rows"] == 11 and s["threads"] >= 128, (N, weff, s)
+
+
+def test_short_lines_of_few_lanes():
+    """Contiguous lines of 105 to 208 points (16 lanes each): divide and conquer up to 160 lanes an SM."""
+    assert hjlo.shape_query(166, 1000, 99)["segment_rows"] < 9
+    assert hjlo.shape_query(166, 2500, 99)["segment_rows"] in (11, 13)

@@ -305,7 +305,7 @@ __device__ __forceinline__ void dense_tile(const CUtensorMap *tmap, const PassPa
         info->kmin = 0x7fffffff;
         info->kmax = (int)0x80000000;
     }
-    if (!stage_tile<T, LAYOUT>(tmap, p, tile, su, kr64, reinterpret_cast<uint64_t *>(smem + p.off_misc))) return;
+    if (!stage_tile<T, LAYOUT, true>(tmap, p, tile, su, kr64, reinterpret_cast<uint64_t *>(smem + p.off_misc))) return;
 
     const int cl = tid >> p.log2lpl, sub = tid & (lpl - 1);
     {

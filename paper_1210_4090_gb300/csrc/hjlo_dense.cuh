@@ -278,8 +278,11 @@ __device__ __noinline__ void dense_leave(const PassParams &p, long long tile)
     search_tile<T, LAYOUT, KALGO_MONGE, OFF>(p, tile);
 }
 
+// `launch`: where p lies in memory (kernel parameters, shared memory), or null
+// for a copy in registers.
 template <typename T, int LAYOUT, typename OFF, int S>
-__device__ __forceinline__ void dense_tile(const CUtensorMap *tmap, const PassParams &p, long long tile)
+__device__ __forceinline__ void dense_tile(const CUtensorMap *tmap, const PassParams &p, long long tile,
+                                           const PassParams *launch)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     T *su = reinterpret_cast<T *>(smem + p.off_u);
@@ -343,8 +346,12 @@ __device__ __forceinline__ void dense_tile(const CUtensorMap *tmap, const PassPa
         __syncthreads();
         if (!info->ok) {
             __syncthreads();                         // everyone has looked
-            const PassParams left = p;
-            dense_leave<T, LAYOUT, OFF>(left, tile);
+            if (launch) {
+                dense_leave<T, LAYOUT, OFF>(*launch, tile);
+            } else {
+                const PassParams left = p;
+                dense_leave<T, LAYOUT, OFF>(left, tile);
+            }
             return;
         }
         const int q = info->q;
@@ -770,7 +777,7 @@ __global__ void __launch_bounds__(dense_threads(S), dense_ctas(S)) pass_kernel_d
     batch_fields(q, it);
     if (q.use_tma && LAYOUT == LAYOUT_STRIDED && threadIdx.x == 0)
         asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(&it->tmap) : "memory");
-    dense_tile<T, LAYOUT, unsigned short, S>(&it->tmap, q, tile);
+    dense_tile<T, LAYOUT, unsigned short, S>(&it->tmap, q, tile, nullptr);
 }
 
 template <typename T, int LAYOUT, int S>
@@ -779,7 +786,7 @@ __global__ void __launch_bounds__(dense_threads(S), dense_ctas(S)) pass_kernel_d
 {
     const long long tile = blockIdx.x;
     if (tile >= p.ntiles) return;
-    dense_tile<T, LAYOUT, unsigned short, S>(&tmap, p, tile);
+    dense_tile<T, LAYOUT, unsigned short, S>(&tmap, p, tile, &p);
 }
 
 }  // namespace hjlo

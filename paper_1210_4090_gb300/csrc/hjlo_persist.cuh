@@ -38,13 +38,13 @@ template <typename T, int LAYOUT>
 __device__ __forceinline__ void persist_tile(const CUtensorMap *tmap, const PassParams &p, long long tile)
 {
     if (p.dense == kFlat)
-        dense_tile<T, LAYOUT, unsigned short, kFlat>(tmap, p, tile);
+        dense_tile<T, LAYOUT, unsigned short, kFlat>(tmap, p, tile, &p);
     else if (p.dense == 9)
-        dense_tile<T, LAYOUT, unsigned short, 9>(tmap, p, tile);
+        dense_tile<T, LAYOUT, unsigned short, 9>(tmap, p, tile, &p);
     else if (p.dense == 13)
-        dense_tile<T, LAYOUT, unsigned short, 13>(tmap, p, tile);
+        dense_tile<T, LAYOUT, unsigned short, 13>(tmap, p, tile, &p);
     else if (p.dense == kWide)
-        dense_tile<T, LAYOUT, unsigned short, kWide>(tmap, p, tile);
+        dense_tile<T, LAYOUT, unsigned short, kWide>(tmap, p, tile, &p);
     else
         pass_tile<T, LAYOUT, KALGO_MONGE>(tmap, p, tile);
 }

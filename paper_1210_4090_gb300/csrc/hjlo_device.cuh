@@ -1165,7 +1165,8 @@ __device__ __forceinline__ void pass_tile(const CUtensorMap *tmap, const PassPar
 // registers, 2048 threads an SM; 300 x 12000 grid, 5 displacements along the
 // strided axis and 1601 along the other: 742 us a step at 58 registers, 690)
 template <typename T, int LAYOUT, int ALGO, typename OFF>
-__global__ void __launch_bounds__(1024, LAYOUT == LAYOUT_STRIDED && ALGO == KALGO_BRUTE ? 2 : 1) pass_kernel(const __grid_constant__ CUtensorMap tmap, PassParams p)
+__global__ void __launch_bounds__(1024, LAYOUT == LAYOUT_STRIDED && ALGO == KALGO_BRUTE ? 2 : 1)
+    pass_kernel(const __grid_constant__ CUtensorMap tmap, PassParams p)
 {
     const long long tile = blockIdx.x;
     if (tile >= p.ntiles) return;

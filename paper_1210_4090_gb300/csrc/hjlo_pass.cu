@@ -368,9 +368,8 @@ static hjlo_status shape_lines(AxisPlan &ax, int esize, int algo, int num_sms, s
 // 2.59 against 2.38 ms) and at most what fits.  `tiles`: for the register-tile
 // searches, whose shared memory is a little more; blocks that do not get them
 // are sized for divide and conquer (shape_launch), which takes 2 (weff - 1)
-// rows of windows above kTwoWindows (one line of 20000 points, 2401
-// displacements: 2400 rows 102 us a pass, 4800 68; 2^18 points, 3801: 3800 rows
-// 267, 7600 184; 8192 points, 1601: 1600 rows 33, 3200 38).
+// rows of windows above kTwoWindows (2^18 points, 3801 displacements: 3800 rows
+// 267 us a pass, 7600 184; 65536 points, 4201: 4200 rows 246, 7529 164).
 // Brute force, whose rows cost weff candidates each
 // against one staged point, also takes blocks for wider windows (up to the
 // full torus window) on an axis with few lines, from one row per block: a

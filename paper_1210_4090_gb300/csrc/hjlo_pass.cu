@@ -261,9 +261,11 @@ static int dense_segment(const AxisPlan &ax, long long NR, long long nlines, int
             if (use > 1.1 * score || nlines * lpl <= 32LL * num_sms) { score = use; best = lpl; }
         }
         // (few lanes with long turns: 900 x 60 grid, 91 displacements 25.6 us a step
-        // against 19.9 by divide and conquer; 278 x 36, 31 displacements 27 against 30)
+        // against 19.9 by divide and conquer; 1000 x 217, 75 displacements 25.2
+        // against 22.2, 400 lines 30.2 against 29.0; 278 x 36, 31 displacements 27
+        // against 30)
         if (sparing && !hinted && (quads + best - 1) / best * ax.weff > 128 && quads > best &&
-            nlines * best < 64LL * num_sms)
+            nlines * best < 200LL * num_sms)
             return 0;
         if (hinted && hint.lpl <= most) best = hint.lpl;
         *lanes = best;

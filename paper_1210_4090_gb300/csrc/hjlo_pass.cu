@@ -231,6 +231,20 @@ static int pivot_group(int weff, int S, int lpl, double *cost)
     return best;
 }
 
+// Whether the flat search gets the row blocks of one line (`rows`: of all its
+// blocks).  Up to 64 rows an SM: 4096 points, 61 displacements 6.2 us a pass, divide
+// and conquer 7.7.  From 512 to 3456 rows: 2^18 points, 95 displacements 11.9 against
+// 13.0, 25 displacements 8.0 against 10.7.  In between it does not fill the SMs
+// (30000 points, 95 displacements 9.4 against 8.0); above, every row at the whole
+// window's cost, rough data makes it the slower one (2^20 points, 95 displacements
+// 21 to 46 us against 24 to 37), as do windows of a few displacements (100000
+// points, 9 displacements 6.7 to 11 against 7.0 to 8.9).
+static bool flat_blocks(long long rows, long long weff, int num_sms)
+{
+    const long long share = rows / num_sms;
+    return weff < 16 ? share < 32 : share < 64 || (share >= 512 && share <= 3456);
+}
+
 // The banded search's kind (rows per segment; hjlo_dense.cuh) and its lanes per
 // line, or 0 for divide and conquer.  `cmin`: the fewest lines a tile can hold;
 // `sparing`: few lanes go to divide and conquer.
@@ -267,6 +281,7 @@ static int dense_segment(const AxisPlan &ax, long long NR, long long nlines, int
         if (sparing && !hinted && (quads + best - 1) / best * ax.weff > 128 && quads > best &&
             nlines * best < 200LL * num_sms)
             return 0;
+        if (!hinted && ax.vblocks > 1 && ax.outer == ax.vblocks && !flat_blocks(NR * nlines, ax.weff, num_sms)) return 0;
         if (hinted && hint.lpl <= most) best = hint.lpl;
         *lanes = best;
         return (quads + best - 1) / best <= 16 ? kFlat : 0;
@@ -376,6 +391,10 @@ static hjlo_status shape_lines(AxisPlan &ax, int esize, int algo, int num_sms, s
 // against one staged point, also takes blocks for wider windows (up to the
 // full torus window) on an axis with few lines, from one row per block: a
 // lone line then spreads over many SMs instead of one SM's binary64 pipe.
+// The flat search's rows cost it the window, which several CTAs an SM hide: blocks of
+// 128 rows, or of the power of two that leaves four an SM (2^18 points, 95
+// displacements: one an SM 16.7 us a pass, blocks of 512 rows 11.9; 500000 points
+// 23.6, of 1024 rows 14.5; 8192 points 8.1, of 128 rows 7.7).
 // A hint (hinted > 0) replaces the share, within [weff - 1 (brute: 1), what
 // fits].
 constexpr int kTwoWindows = 2048;
@@ -398,6 +417,8 @@ static long long block_rows(const AxisPlan &ax, int esize, int algo, int num_sms
     if (brute && 4 * w > N && !(2 * lines < num_sms)) return 0;     // wide windows: few lines only
     long long vR = brute ? 1 : (!tiles && w > kTwoWindows) ? 2 * (w - 1) : w - 1;
     vR = std::max(vR, (N * lines + num_sms - 1) / num_sms);
+    if (tiles && w <= kFlatMaxWindow)
+        for (vR = 128; vR * 4 * num_sms < N * lines;) vR *= 2;
     if (hinted > 0) vR = std::max(hinted, least);
     vR = std::min(vR, fit_pts - (w - 1));
     vR = std::min(vR, N - (w - 1));                                 // a block never spans the line

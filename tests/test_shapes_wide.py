@@ -74,3 +74,14 @@ def test_short_lines_of_few_lanes():
     """Contiguous lines of 105 to 208 points (16 lanes each): divide and conquer up to 160 lanes an SM."""
     assert hjlo.shape_query(166, 1000, 99)["segment_rows"] < 9
     assert hjlo.shape_query(166, 2500, 99)["segment_rows"] in (11, 13)
+
+
+# the flat search's blocks are of a power of two of rows, divide and conquer's hold an SM's share
+@pytest.mark.parametrize("N,lines,weff,rows", [
+    (4096, 1, 61, 128), (9600, 1, 95, 128), (30000, 1, 95, 198),      # a few rows an SM; too few to fill it
+    (78000, 1, 95, 256), (1 << 18, 1, 95, 512), (500000, 1, 25, 1024),   # four blocks an SM at most
+    (1 << 20, 1, 95, 6899), (100000, 1, 9, 658),          # the whole window's cost; a few displacements
+    (900, 60, 91, 128), (20000, 16, 81, 1024)])           # several lines
+def test_flat_row_blocks(N, lines, weff, rows):
+    s = hjlo.shape_query(N, lines, weff)
+    assert s["block_rows"] == rows and s["row_blocks"] > 1, s

@@ -257,7 +257,7 @@ static bool flat_blocks(long long rows, long long weff, int num_sms)
 // the first in registers, 9 or 13 rows a segment; a power of two of lanes then
 // leaves at most 30 % of them idle, and a pivot scans the whole window, weff / 9
 // add-minimums and shared-memory words a row, which bounds the windows.
-static int dense_segment(const AxisPlan &ax, long long NR, long long nlines, int cmin, int num_sms,
+static int dense_segment(const AxisPlan &ax, int esize, long long NR, long long nlines, int cmin, int num_sms,
                          const ShapeHints &hint, bool sparing, int *lanes)
 {
     if (ax.weff > kDenseMaxWindow) return 0;
@@ -277,8 +277,9 @@ static int dense_segment(const AxisPlan &ax, long long NR, long long nlines, int
         // (few lanes with long turns: 900 x 60 grid, 91 displacements 25.6 us a step
         // against 19.9 by divide and conquer; 1000 x 217, 75 displacements 25.2
         // against 22.2, 400 lines 30.2 against 29.0; 278 x 36, 31 displacements 27
-        // against 30)
-        if (sparing && !hinted && (quads + best - 1) / best * ax.weff > 128 && quads > best &&
+        // against 30; binary32 strided tiles, of four lines at least, stay: 304 x 299
+        // grid, 69 displacements 17.9 against 20.2)
+        if (sparing && !hinted && (ax.inner == 1 || esize == 8) && (quads + best - 1) / best * ax.weff > 128 && quads > best &&
             nlines * best < 200LL * num_sms)
             return 0;
         if (!hinted && ax.vblocks > 1 && ax.outer == ax.vblocks && !flat_blocks(NR * nlines, ax.weff, num_sms)) return 0;
@@ -310,8 +311,15 @@ static int dense_segment(const AxisPlan &ax, long long NR, long long nlines, int
     // displacements 29.8 against 45.5, 2001 34.7 against 98.
     // Contiguous lines with 16 lanes: 1000 x 166 grid, 99 displacements 25.6 us a
     // step against 22.5, 1500 x 208 grid 30.9 against 26.6, 1000 x 130 21.3 against
-    // 22.1.
-    long long few = ax.inner == 1 && lpl == 16 ? 160 : 100;
+    // 22.1; with 32 lanes: 752 x 250 grid, 153 displacements 26.6 against 21.4, 1000
+    // x 360, 191 displacements 25.4 against 21.3; binary32, 759 x 245 grid, 169
+    // displacements 31.5 against 28.4.  Strided axes, whose tiles of two lines
+    // and more share a CTA: 425 x 172 grid, 101 displacements 46.6 a step of the
+    // gradients against 52.3, 539 x 103, 123 displacements 15.5 against 18.1.
+    long long few = 100;
+    if (ax.inner == 1 && lpl == 16) few = 160;
+    if (ax.inner == 1 && lpl == 32 && NR < 384) few = 250;
+    if (ax.inner != 1 && lpl >= 32) few = lpl == 32 ? 64 : 32;
     if (!sparing || lpl >= 128 || ax.weff > 480) few = 64;
     if (wide) few = ax.weff > 640 ? 0 : 32;
     if (!hinted && nlines * lpl < few * num_sms) return 0;
@@ -500,7 +508,7 @@ static hjlo_status shape_lines(AxisPlan &ax, int esize, int algo, int num_sms, s
 
     // rows searched per line (a row block searches only its own rows)
     const long long NR = (ax.rows > 0 && ax.rows < N) ? ax.rows : N;
-    ax.dense = (algo == KALGO_MONGE) ? dense_segment(ax, NR, nlines, cmin, num_sms, hint, sparing, &ax.lpl)
+    ax.dense = (algo == KALGO_MONGE) ? dense_segment(ax, esize, NR, nlines, cmin, num_sms, hint, sparing, &ax.lpl)
                                      : 0;
     if (ax.dense) {
         ax.log2lpl = ilog2(ax.lpl);

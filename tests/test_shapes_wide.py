@@ -85,3 +85,11 @@ def test_short_lines_of_few_lanes():
 def test_flat_row_blocks(N, lines, weff, rows):
     s = hjlo.shape_query(N, lines, weff)
     assert s["block_rows"] == rows and s["row_blocks"] > 1, s
+
+
+@pytest.mark.parametrize("esize", [8, 4])
+def test_lines_of_32_lanes(esize):
+    """Contiguous lines of 209 to 383 points (32 lanes each): divide and conquer up to 250 lanes an SM."""
+    assert hjlo.shape_query(250, 752, 153, esize)["segment_rows"] < 9
+    assert hjlo.shape_query(250, 1400, 153, esize)["segment_rows"] in (9, 13)
+    assert hjlo.shape_query(414, 1000, 99, esize)["segment_rows"] in (9, 13)
